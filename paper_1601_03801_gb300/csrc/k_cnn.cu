@@ -246,8 +246,9 @@ size_t cnn_param_count() { return kNP; }
 
 size_t cnn_work_bytes(int64_t n) {
   // x(bf16x4) a1,a2(bf16x32) y(f32x4) g_y(f32x4) g2,g1(f32x32) + packed weights
+  // (and up to 255 bytes of alignment for each of the 17 parts)
   return (size_t)n * (8 + 64 + 64 + 16 + 16 + 128 + 128) + 8 * kNP * sizeof(float) + 1024 +
-         27 * 32 * 32 * 2 + (size_t)kWgBlocks * (27 * 1024 + 32) * 4 + 1024;
+         27 * 32 * 32 * 2 + (size_t)kWgBlocks * (27 * 1024 + 32) * 4 + 1024 + 17 * 256;
 }
 
 struct CnnBufs {
@@ -259,26 +260,33 @@ struct CnnBufs {
   float* bpart;          // [kWgBlocks][32] bias-gradient partials
 };
 
+// Every part starts on a 256-byte boundary: the kernels read some of them as 16-byte words,
+// and the parts before them have an odd number of 8-byte words on a mesh of odd size.
 static CnnBufs carve(void* work, int64_t n) {
   char* p = (char*)work;
+  auto take = [&](size_t bytes) {
+    void* at = p;
+    p += (bytes + 255) & ~(size_t)255;
+    return at;
+  };
   CnnBufs b;
-  b.x = (__nv_bfloat16*)p; p += n * 8;
-  b.a1 = (__nv_bfloat16*)p; p += n * 64;
-  b.a2 = (__nv_bfloat16*)p; p += n * 64;
-  b.y = (float*)p; p += n * 16;
-  b.gy = (float*)p; p += n * 16;
-  b.g2 = (float*)p; p += n * 128;
-  b.g1 = (float*)p; p += n * 128;
-  b.wf1 = (float*)p; p += 32 * 4 * 27 * 4;
-  b.wb1 = (float*)p; p += 32 * 4 * 27 * 4;
-  b.wf2 = (float*)p; p += 32 * 32 * 27 * 4;
-  b.wb2 = (float*)p; p += 32 * 32 * 27 * 4;
-  b.wf3 = (float*)p; p += 4 * 32 * 27 * 4;
-  b.wb3 = (float*)p; p += 4 * 32 * 27 * 4;
-  b.bias_r = (float*)p; p += 128 * 4;
-  b.w2mma = (__nv_bfloat16*)p; p += 27 * 32 * 32 * 2;
-  b.wpart = (float*)p; p += (size_t)kWgBlocks * 27 * 1024 * 4;
-  b.bpart = (float*)p;
+  b.x = (__nv_bfloat16*)take(n * 8);
+  b.a1 = (__nv_bfloat16*)take(n * 64);
+  b.a2 = (__nv_bfloat16*)take(n * 64);
+  b.y = (float*)take(n * 16);
+  b.gy = (float*)take(n * 16);
+  b.g2 = (float*)take(n * 128);
+  b.g1 = (float*)take(n * 128);
+  b.wf1 = (float*)take(32 * 4 * 27 * 4);
+  b.wb1 = (float*)take(32 * 4 * 27 * 4);
+  b.wf2 = (float*)take(32 * 32 * 27 * 4);
+  b.wb2 = (float*)take(32 * 32 * 27 * 4);
+  b.wf3 = (float*)take(4 * 32 * 27 * 4);
+  b.wb3 = (float*)take(4 * 32 * 27 * 4);
+  b.bias_r = (float*)take(128 * 4);
+  b.w2mma = (__nv_bfloat16*)take(27 * 32 * 32 * 2);
+  b.wpart = (float*)take((size_t)kWgBlocks * 27 * 1024 * 4);
+  b.bpart = (float*)take((size_t)kWgBlocks * 32 * 4);
   return b;
 }
 
