@@ -216,8 +216,8 @@ void sedi_default_params(sedi_params* p);
    Hertz contact time; the caller chooses dt.)  *out is owned by the caller and
    released with sedi_destroy.  Errors: EINVAL, ENOMEM, ECUDA.  The environment
    variable SEDI_BARRIER_SPIN_LIMIT, read here, lowers the number of polls after
-   which a wait at the grid-wide barrier of the smoother (meshes too large for one
-   thread-block cluster) gives up and the averaging returns SEDI_ETIMEOUT (default
+   which a wait between the smoother's thread blocks (meshes too large for one
+   thread-block cluster or block) gives up and the averaging returns SEDI_ETIMEOUT (default
    2^22, about 0.3 s); it exists so tests can make that wait run out. */
 int sedi_create(const sedi_params* p, sedi_handle** out);
 void sedi_destroy(sedi_handle* h);
@@ -416,7 +416,7 @@ int sedi_get_stats(sedi_handle* h, sedi_stats* out);
  *   msg     : optional host buffer of msg_len bytes for an error message.
  * Limit: 8 * C <= SEDI_STATIC_MAX_WORDS, i.e. up to 131,072 cells with any
  * n_fields <= 8 (the solver keeps 8 words per cell); larger meshes return
- * SEDI_EINVAL.  The scratch (about 50 MB) lives on every GPU that loads the
+ * SEDI_EINVAL.  The scratch (about 54 MB) lives on every GPU that loads the
  * library until the process exits.  Every call looks up the scratch's device
  * address on the current device (cudaGetSymbolAddress, which allocates nothing).
  * The call copies its status to the host and synchronises its stream, so it must

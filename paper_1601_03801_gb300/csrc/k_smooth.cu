@@ -1036,6 +1036,820 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
   }
 }
 
+// ---------------------------------------------------------------- resident solver
+// A group of CTAs solves one (mesh, field) pair at a time with the whole field on chip:
+// CTA (ix, iy, iz) of the group holds a brick of bx x by x bz cells.
+// x (wide) and the recursive residual q live in registers (a thread owns chunks of
+// kRsZ cells along z), the direction d in shared memory, double-buffered, with halos.
+// Same iteration, and the same FP32 recursion per cell, as the grid solver above: only
+// the association of the sums of a round and the low bits of the true residual differ.
+// Halos between CTAs go through global memory (they stay in L2) as 8-byte words of a value
+// and the exchange's number, so a receiver polls the data itself: no fence, no flag and no
+// barrier between a store and its use.  A round's sums travel the same way.  Every wait is
+// bounded and every CTA of a group resident (cooperative launch); a field in one CTA
+// needs neither.  Several groups work on the mesh's fields at once when they fit.
+// A missing face (zero flux) is a halo that repeats the boundary cell: its difference is
+// exactly zero, so there are no per-face branches.
+//
+// A direction buffer: the chunks [zc][y + 1][x + 1] as 4-cell vectors, with a halo chunk
+// on each x and y side (an odd number a row, so a column of chunks meets no bank twice),
+// then the planes below and above the brick, [y][x] words each, where z is cut.  A step
+// reads a chunk and its four neighbours as vectors and two more words: 7 loads for 4
+// cells.  A cut across z costs a word a cell of halo traffic, one across x or y a vector
+// for four, so z is cut last.
+//
+// What bounds it: the exchange and the issue of a step.  On 128 x 64 x 128 a step takes
+// 7.3 us for 6,900 cells a CTA, of which the FP32 pipe accounts for 0.9 us (29 operations
+// a cell at 128 a clock and SM; packed f32x2 instructions run at the same operation rate),
+// one way between SMs through L2 for 0.8 us.
+// Seven fields of random values, microseconds a call, streaming grid solver -> here:
+// 128 x 64 x 128 9,790 -> 4,960, 256 x 128 x 64 10,190 -> 5,590, 96 x 96 x 24
+// 2,020 -> 980; 10 x 10 x 20 in one CTA 440 -> 200; FP64 19 x 15 x 31 4,400 -> 710 (the
+// streaming solver ran it on 35 blocks).
+constexpr int kRsZ = 4;              // cells of a chunk
+constexpr int kRsMaxGroup = 160;     // CTAs of a group at most
+constexpr size_t kRsSmem = 176 * 1024;  // dynamic shared memory of a CTA at most
+
+// Threads of a CTA, and the chunks a thread holds at most: their x and q are 12 registers
+// each in the double-float form (16 in FP64) of the 128 it has.
+constexpr int kRsThreads = 512;
+constexpr int kRsChunks = 4;         // where they do, and in FP64
+constexpr int kRsChunksBig = 7;      // larger meshes
+
+// Sums of a round: FP32 residuals add up compensated (double-float), so a thread may sum
+// many cells, and a warp stays off the narrow FP64 pipe.
+struct SumF {
+  dd v;
+  __device__ void add(float x) { v = dd_add_f(v, x); }
+  __device__ void join(int o) {
+    v = dd_add(v, dd{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+  }
+  __device__ void plus(const SumF& o) { v = dd_add(v, o.v); }
+  // a reduce-scatter step: keep one of two sums (b where up), added to the partner's
+  __device__ static SumF give(const SumF& a, const SumF& b, bool up, int o) {
+    const dd keep = up ? b.v : a.v, out = up ? a.v : b.v;
+    return SumF{dd_add(keep, dd{__shfl_xor_sync(0xffffffffu, out.hi, o), __shfl_xor_sync(0xffffffffu, out.lo, o)})};
+  }
+  __device__ double d() const { return dd_to_double(v); }
+};
+struct SumD {
+  double v;
+  __device__ void add(double x) { v += x; }
+  __device__ void join(int o) { v += __shfl_xor_sync(0xffffffffu, v, o); }
+  __device__ void plus(const SumD& o) { v += o.v; }
+  __device__ static SumD give(const SumD& a, const SumD& b, bool up, int o) {
+    return SumD{(up ? b.v : a.v) + __shfl_xor_sync(0xffffffffu, up ? a.v : b.v, o)};
+  }
+  __device__ double d() const { return v; }
+};
+
+// The four cells of a chunk as loaded from a direction buffer.
+struct C4f {
+  float v[kRsZ];
+};
+struct C4d {
+  double v[kRsZ];
+};
+__device__ __forceinline__ C4f ld_chunk(const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  return C4f{{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ C4d ld_chunk(const double* p) {
+  const double2 t = reinterpret_cast<const double2*>(p)[0], u = reinterpret_cast<const double2*>(p)[1];
+  return C4d{{t.x, t.y, u.x, u.y}};
+}
+__device__ __forceinline__ void st_chunk(float* p, const float (&v)[kRsZ]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st_chunk(double* p, const double (&v)[kRsZ]) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+}
+
+// x as it is published for the true residual: the double-float word split over the two
+// direction buffers, the other words in the first.
+template <class T>
+struct Pub;
+template <>
+struct Pub<dd> {
+  static constexpr int n = 2;
+  __device__ static float word(dd v, int k) { return k ? v.lo : v.hi; }
+  __device__ static dd one(const float* d0, const float* d1, int o) { return dd{d0[o], d1[o]}; }
+  __device__ static void chunk(const float* d0, const float* d1, int o, dd (&t)[kRsZ]) {
+    const C4f h = ld_chunk(d0 + o), l = ld_chunk(d1 + o);
+#pragma unroll
+    for (int z = 0; z < kRsZ; ++z) t[z] = dd{h.v[z], l.v[z]};
+  }
+};
+template <class T>
+struct Pub {
+  static constexpr int n = 1;
+  __device__ static T word(T v, int) { return v; }
+  __device__ static T one(const T* d0, const T*, int o) { return d0[o]; }
+  __device__ static void chunk(const T* d0, const T*, int o, T (&t)[kRsZ]) {
+    const auto h = ld_chunk(d0 + o);
+#pragma unroll
+    for (int z = 0; z < kRsZ; ++z) t[z] = h.v[z];
+  }
+};
+
+// True residual b - A x of a cell (wide) as the narrow word: c the cell, l r f k its x and
+// y neighbours, dn up its planes; cz the z-face coefficients of a graded mesh.
+template <class T>
+struct Resid {
+  using W = Wide<T>;
+  using N = typename W::N;
+  __device__ static T pair(T m, T p, T c) { return W::addq(W::subq(m, c), W::subq(p, c)); }
+  __device__ static N eval(const T (&cf)[3], T c, T l, T r, T f, T k, T dn, T up, T b) {
+    const T lap = W::addq(W::addq(W::mul(cf[0], pair(l, r, c)), W::mul(cf[1], pair(f, k, c))),
+                          W::mul(cf[2], pair(dn, up, c)));
+    return W::narrow(W::subq(b, W::subq(c, lap)));
+  }
+  __device__ static N eval_z(const T (&cf)[3], const double* cz, T c, T l, T r, T f, T k, T dn, T up, T b) {
+    T lap = W::addq(W::mul(cf[0], pair(l, r, c)), W::mul(cf[1], pair(f, k, c)));
+    lap = W::addq(lap, W::mul(W::from_d(cz[0]), W::subq(dn, c)));
+    lap = W::addq(lap, W::mul(W::from_d(cz[1]), W::subq(up, c)));
+    return W::narrow(W::subq(b, W::subq(c, lap)));
+  }
+};
+// Double-float: the high words go through error-free sums and products, every error and
+// low word is collected in one FP32 sum, and nothing is renormalised on the way (98
+// operations a cell instead of 165; its error, a few 2^-47 of |x|, is below that of the
+// renormalising additions, 2^-44).
+template <>
+struct Resid<dd> {
+  // cf * ((m - c) + (p - c)) as an unnormalised pair
+  __device__ static dd axis(dd cf, dd m, dd p, dd c) {
+    const dd s = two_sum(m.hi, p.hi);
+    const dd t = two_sum(s.hi, -2.0f * c.hi);
+    const float lo = (s.lo + t.lo) + ((m.lo + p.lo) - 2.0f * c.lo);
+    const dd q = two_prod(cf.hi, t.hi);
+    return dd{q.hi, __fmaf_rn(cf.hi, lo, __fmaf_rn(cf.lo, t.hi, q.lo))};
+  }
+  __device__ static dd face(dd cf, dd m, dd c) {
+    const dd t = two_sum(m.hi, -c.hi);
+    const dd q = two_prod(cf.hi, t.hi);
+    return dd{q.hi, __fmaf_rn(cf.hi, t.lo + (m.lo - c.lo), __fmaf_rn(cf.lo, t.hi, q.lo))};
+  }
+  __device__ static dd plus(dd a, dd b) {  // unnormalised
+    const dd s = two_sum(a.hi, b.hi);
+    return dd{s.hi, s.lo + (a.lo + b.lo)};
+  }
+  __device__ static float eval(const dd (&cf)[3], dd c, dd l, dd r, dd f, dd k, dd dn, dd up, dd b) {
+    const dd lap = plus(plus(axis(cf[0], l, r, c), axis(cf[1], f, k, c)), axis(cf[2], dn, up, c));
+    const dd v = plus(plus(b, dd{-c.hi, -c.lo}), lap);
+    return __fadd_rn(v.hi, v.lo);
+  }
+  __device__ static float eval_z(const dd (&cf)[3], const double* cz, dd c, dd l, dd r, dd f, dd k, dd dn, dd up,
+                                 dd b) {
+    const dd xy = plus(axis(cf[0], l, r, c), axis(cf[1], f, k, c));
+    const dd zz = plus(face(dd_from_double(cz[0]), dn, c), face(dd_from_double(cz[1]), up, c));
+    const dd v = plus(plus(b, dd{-c.hi, -c.lo}), plus(xy, zz));
+    return __fadd_rn(v.hi, v.lo);
+  }
+};
+
+// Words that carry their own arrival: each 8-byte word of global memory holds 32 bits of
+// data and the number of the exchange that wrote it.  A 64-bit access is indivisible, so
+// a reader that finds the number has the data, with no fence between them.
+__device__ __forceinline__ unsigned long long tag(uint32_t w, uint32_t e) {
+  return (unsigned long long)e << 32 | w;
+}
+__device__ __forceinline__ void put2(unsigned long long* p, uint32_t w0, uint32_t w1, uint32_t e) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(tag(w0, e)), "l"(tag(w1, e)) : "memory");
+}
+__device__ __forceinline__ void put1(unsigned long long* p, uint32_t w, uint32_t e) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(tag(w, e)) : "memory");
+}
+struct Tag2 {
+  unsigned long long a, b;
+  __device__ void load(const unsigned long long* p) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  }
+  __device__ bool is(uint32_t e) const { return (uint32_t)(a >> 32) == e && (uint32_t)(b >> 32) == e; }
+};
+__device__ __forceinline__ unsigned long long get1(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+// A waiting poll: false once the limit is reached (SEDI_ETIMEOUT recorded) or another
+// block gave up.
+struct Spin {
+  unsigned n = 0;
+  __device__ bool go(Ctl* ctl, long long limit) {
+    if (++n > (unsigned)limit) {
+      atomicCAS((int*)&ctl->cg_status, 0, SEDI_ETIMEOUT);
+      return false;
+    }
+    return (n & 255) != 0 || *((volatile int*)&ctl->cg_status) != SEDI_ETIMEOUT;
+  }
+};
+__device__ __forceinline__ uint32_t as_word(float v, int) { return __float_as_uint(v); }
+__device__ __forceinline__ uint32_t as_word(double v, int k) {
+  return k ? (uint32_t)__double2hiint(v) : (uint32_t)__double2loint(v);
+}
+__device__ __forceinline__ void of_words(float& v, uint32_t a, uint32_t) { v = __uint_as_float(a); }
+__device__ __forceinline__ void of_words(double& v, uint32_t a, uint32_t b) { v = __hiloint2double((int)b, (int)a); }
+
+// The halos of a CTA from its tagged words: unit u < nu a chunk (kRsZ values), the nw units
+// after them one value each, laid out in that order; pull[u] the word of the buffer that
+// it fills (top bit: none).  Not inlined: a caller full of live registers would spill.
+template <class N, int TH>
+__device__ __noinline__ bool rs_receive(N* D, const uint32_t* pull, int nu, int nw, const unsigned long long* src,
+                                        uint32_t seq, Ctl* ctl, long long spin_limit) {
+  constexpr int NW = sizeof(N) / 4, K = 2;  // chunks in flight
+  bool ok = true;
+#pragma unroll 1
+  for (int u0 = threadIdx.x; u0 < nu; u0 += K * TH) {
+#pragma unroll
+    for (int h = 0; h < NW; ++h) {  // FP64: two halves of a chunk
+      Tag2 t[K][2];
+      uint32_t e[K];
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        const int u = u0 + q * TH;
+        e[q] = u < nu ? pull[u] : 1u << 31;
+        if (e[q] >> 31) continue;
+        t[q][0].load(src + (u * NW + h) * 4);
+        t[q][1].load(src + (u * NW + h) * 4 + 2);
+      }
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        if (e[q] >> 31) continue;
+        Spin spin;
+        while (!(t[q][0].is(seq) && t[q][1].is(seq)) && ok) {
+          ok = spin.go(ctl, spin_limit);
+          const int u = u0 + q * TH;
+          t[q][0].load(src + (u * NW + h) * 4);
+          t[q][1].load(src + (u * NW + h) * 4 + 2);
+        }
+        N* const to = D + e[q];
+        if constexpr (NW == 1) {
+          N c[kRsZ];
+          of_words(c[0], (uint32_t)t[q][0].a, 0u);
+          of_words(c[1], (uint32_t)t[q][0].b, 0u);
+          of_words(c[2], (uint32_t)t[q][1].a, 0u);
+          of_words(c[3], (uint32_t)t[q][1].b, 0u);
+          st_chunk(to, c);
+        } else {
+          of_words(to[2 * h], (uint32_t)t[q][0].a, (uint32_t)t[q][0].b);
+          of_words(to[2 * h + 1], (uint32_t)t[q][1].a, (uint32_t)t[q][1].b);
+        }
+      }
+    }
+  }
+  const unsigned long long* const ws = src + (size_t)nu * kRsZ * NW;
+#pragma unroll 1
+  for (int u0 = threadIdx.x; u0 < nw; u0 += 4 * TH) {
+    unsigned long long t[4][NW];
+    uint32_t e[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int u = u0 + q * TH;
+      e[q] = u < nw ? pull[nu + u] : 1u << 31;
+      if (!(e[q] >> 31))
+#pragma unroll
+        for (int k = 0; k < NW; ++k) t[q][k] = get1(ws + u * NW + k);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (e[q] >> 31) continue;
+#pragma unroll
+      for (int k = 0; k < NW; ++k) {
+        Spin spin;
+        while ((uint32_t)(t[q][k] >> 32) != seq && ok) {
+          ok = spin.go(ctl, spin_limit);
+          t[q][k] = get1(ws + (u0 + q * TH) * NW + k);
+        }
+      }
+      of_words(D[e[q]], (uint32_t)t[q][0], (uint32_t)t[q][NW - 1]);
+    }
+  }
+  return ok;
+}
+
+template <class T, bool GR, int M>
+__global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
+  using W = Wide<T>;
+  using N = typename W::N;
+  using P = Pub<T>;
+  using Sum = typename std::conditional<sizeof(N) == 8, SumD, SumF>::type;
+  constexpr int TH = kRsThreads, kWarps = TH / 32;
+  constexpr int NW = sizeof(N) / 4;  // 32-bit words of a narrow value
+  // a chunk's first word: index of its first cell, valid cells, chunk along z; its second
+  // word: the indexes of the cells below and above it
+  constexpr int kCnt = 18, kZc = 21;
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  __shared__ double s_part[kRsMaxGroup][kQ];  // every CTA's sums
+  __shared__ Sum s_red[kWarps][kQ];
+  __shared__ double s_tot[kQ], s_shift;
+  __shared__ uint2 s_info[M * TH];
+  __shared__ int s_cell[M * TH];  // first cell of a chunk in the mesh
+  __shared__ int s_k, s_zero, s_ok;
+  // the item's neighbours and pointers (registers hold the field)
+  __shared__ struct {
+    int nb[6];             // neighbour CTAs below / above along x, y and z (-1: none)
+    int dst[6];            // x, y: words from a boundary cell to the halo that takes it;
+                           // z: the halo plane that takes it
+    T *x, *b, *xp;
+    const T* guess;
+    N* r;                  // the narrow true residual between its pass and the step loop
+    unsigned long long* halo;  // grid: the group's tagged halo words, [CTA][parity][channel][hw]
+    unsigned long long* sums;  // grid: the group's tagged sums, [parity][CTA][kQ][2]
+    double inv;            // 1 / cells, or 1 / total weight on a graded mesh
+  } s_g;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int G = a.rs_G, rank = (int)(blockIdx.x % (unsigned)G);
+  const int64_t grp = blockIdx.x / (unsigned)G, ngrp = gridDim.x / (unsigned)G;
+  uint32_t seq = 0, rseq = 0;  // halo exchanges and reductions so far
+  if (tid == 0) s_ok = 1;
+  const int64_t items = (int64_t)a.B * a.nf;
+  for (int64_t w = grp; w < items; w += ngrp) {
+    const int bi = (int)(w / a.nf), f = (int)(w % a.nf);
+    const SmoothMeshDev& md = a.mesh[bi];
+    const int64_t C = md.C;
+    const int nx = md.nc[0], ny = md.nc[1], nz = md.nc[2], nxy = nx * ny;
+    const int px = md.rs_px, py = md.rs_py, pz = md.rs_pz;
+    const int ix = rank % px, iy = rank / px % py, iz = rank / (px * py);
+    // first cell of part i of n cells cut in p
+    auto cut = [](int i, int n, int p) { return (int)((int64_t)i * n / p); };
+    const int x0 = cut(ix, nx, px), bx = cut(ix + 1, nx, px) - x0;
+    const int y0 = cut(iy, ny, py), by = cut(iy + 1, ny, py) - y0;
+    const int z0 = cut(iz, nz, pz), bz = cut(iz + 1, nz, pz) - z0;
+    const int bxm = (nx + px - 1) / px, bym = (ny + py - 1) / py;
+    const int nzcm = ((nz + pz - 1) / pz + kRsZ - 1) / kRsZ;
+    const bool zcut = pz > 1 || md.per[2];              // halo planes are exchanged
+    const int pr = ((bxm + 2) | 1) * kRsZ;              // words of a row
+    const int cs = (bym + 2) * pr;                      // words of a chunk layer
+    const int zlo = nzcm * cs, zhi = zlo + (zcut ? bym * bxm : 0);   // halo planes
+    const int words = (zhi + (zcut ? bym * bxm : 0) + 3) & ~3;      // of a buffer
+    const int bxy = bx * by, nzc = (bz + kRsZ - 1) / kRsZ, nch = bxy * nzc;
+    const bool part = bz % kRsZ != 0;
+    // grid: room for the halo words of a CTA and channel
+    const int hw = 2 * (nzcm * kRsZ * (bxm + bym) + (zcut ? bxm * bym : 0));
+    const int nu = 2 * nzc * (bx + by), nw = zcut ? 2 * bxy : 0;  // halo units: chunks, words
+    N* const D0 = (N*)s_dyn;
+    N* const D1 = D0 + words;
+    N* const s_cz = D1 + words;  // [bz][2] z-face coefficients (graded mesh)
+    // halo units: {word of the boundary cell | kLocal, target}: a word of this CTA's buffer
+    // (local) or a tagged word of the neighbour's; and the word of this CTA's halo that
+    // unit u of its own tagged words fills (kLocal: none)
+    uint2* const s_push = (uint2*)(s_cz + (GR ? 2 * nzcm * kRsZ : 0));
+    uint32_t* const s_pull = (uint32_t*)(s_push + 2 * nzcm * (bxm + bym) + (zcut ? 2 * bxm * bym : 0));
+    constexpr uint32_t kLocal = 1u << 31;
+
+    __syncthreads();  // the previous item's readers of s_g and s_info are done
+    if (tid == 0) {
+      auto rank_of = [&](int jx, int jy, int jz) { return (jz * py + jy) * px + jx; };
+      // the neighbour on each side, or -1 at a face without flux; a missing x or y face
+      // pushes the boundary cells to this CTA's own halo on that side, a missing z face
+      // needs none (the cell below or above is the boundary cell itself)
+      const int p3[3] = {px, py, pz};
+      for (int s = 0; s < 6; ++s) {
+        const int ax = s >> 1, up = s & 1;
+        int j[3] = {ix, iy, iz};
+        j[ax] += up ? 1 : -1;
+        const bool in = j[ax] >= 0 && j[ax] < p3[ax];
+        if (!in) j[ax] = up ? 0 : p3[ax] - 1;
+        s_g.nb[s] = in || md.per[ax] ? rank_of(j[0], j[1], j[2]) : -1;
+        const int n = ax == 0 ? nx : ny, mine = ax == 0 ? bx : by, step = ax == 0 ? kRsZ : pr;
+        if (ax < 2) {
+          const int theirs = cut(j[ax] + 1, n, p3[ax]) - cut(j[ax], n, p3[ax]);
+          s_g.dst[s] = s_g.nb[s] < 0 ? (up ? step : -step) : (up ? -mine * step : theirs * step);
+        } else {
+          s_g.dst[s] = up ? zlo : zhi;
+        }
+      }
+      s_g.x = (T*)md.x + f * C;
+      s_g.b = (T*)md.b + f * C;
+      s_g.xp = md.xp ? (T*)md.xp + f * C : nullptr;
+      s_g.guess = md.guess ? (const T*)md.guess + f * C : nullptr;
+      s_g.r = (N*)md.q + f * C;
+      s_g.inv = GR ? 1.0 / md.z.wsum : 1.0 / (double)C;
+      s_g.sums = (unsigned long long*)md.d[0] + (size_t)grp * G * 2 * kQ * 2;
+      s_g.halo = (unsigned long long*)md.d[0] + (size_t)ngrp * G * 2 * kQ * 2 + (size_t)grp * G * 2 * P::n * hw * NW;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int m = 0; m < M; ++m) {
+      const int c = tid + m * TH;
+      uint2 in = make_uint2(0u, 0u);
+      int g = 0;
+      if (c < nch) {
+        const int zc = c / bxy, r = c - zc * bxy, y = r / bx, x = r - y * bx;
+        const int cnt = bz - zc * kRsZ < kRsZ ? bz - zc * kRsZ : kRsZ;
+        const int o = zc * cs + (y + 1) * pr + (x + 1) * kRsZ;
+        const int ob = zc > 0 ? o - cs + kRsZ - 1 : s_g.nb[4] < 0 ? o : zlo + r;
+        const int oa = zc + 1 < nzc ? o + cs : s_g.nb[5] < 0 ? o + cnt - 1 : zhi + r;
+        in.x = (uint32_t)o | ((uint32_t)cnt << kCnt) | ((uint32_t)zc << kZc);
+        in.y = (uint32_t)ob | ((uint32_t)oa << 16);
+        g = (z0 + zc * kRsZ) * nxy + (y0 + y) * nx + x0 + x;
+      }
+      s_info[m * TH + tid] = in;
+      s_cell[m * TH + tid] = g;
+    }
+    // the first unit of side s in CTA r of the group (its units are in side order); words
+    // of the z sides follow the chunks
+    [[maybe_unused]] auto ufirst = [&](int s, int r) {
+      const int jx = r % px, jy = r / px % py, jz = r / (px * py);
+      const int wx = cut(jx + 1, nx, px) - cut(jx, nx, px), wy = cut(jy + 1, ny, py) - cut(jy, ny, py);
+      const int wz = (cut(jz + 1, nz, pz) - cut(jz, nz, pz) + kRsZ - 1) / kRsZ;
+      const int c = s < 2 ? s * wz * wy : 2 * wz * wy + (s == 2 ? 0 : wz * wx);
+      return s < 4 ? c * kRsZ : 2 * wz * (wx + wy) * kRsZ + (s - 4) * wx * wy;
+    };
+    // the halo units
+    for (int u = tid; u < nu + nw; u += TH) {
+      int s, v, src, dst, fill, far;
+      if (u < nu) {
+        const int nxs = nzc * by, nys = nzc * bx;
+        s = u < nxs ? 0 : u < 2 * nxs ? 1 : u < 2 * nxs + nys ? 2 : 3;
+        v = u - (s == 0 ? 0 : s == 1 ? nxs : s == 2 ? 2 * nxs : 2 * nxs + nys);
+        const int wide = s < 2 ? by : bx, zc = v / wide, i = v - zc * wide, step = s < 2 ? pr : kRsZ;
+        const int base = zc * cs + pr + kRsZ + i * step;
+        src = base + (s == 1 ? (bx - 1) * kRsZ : s == 3 ? (by - 1) * pr : 0);
+        fill = base + (s == 0 ? -kRsZ : s == 1 ? bx * kRsZ : s == 2 ? -pr : by * pr);
+        dst = src + s_g.dst[s];
+        far = s_g.nb[s] < 0 ? 0 : ufirst(s ^ 1, s_g.nb[s]) + v * (u < nu ? kRsZ : 1);
+      } else {
+        s = u - nu < bxy ? 4 : 5;
+        v = u - nu - (s == 5 ? bxy : 0);
+        const int y = v / bx;
+        src = (s == 5 ? (bz - 1) / kRsZ * cs + (bz - 1) % kRsZ : 0) + (y + 1) * pr + (v - y * bx + 1) * kRsZ;
+        fill = (s == 5 ? zhi : zlo) + v;
+        dst = s_g.dst[s] + v;
+        far = s_g.nb[s] < 0 ? 0 : ufirst(s ^ 1, s_g.nb[s]) + v * (u < nu ? kRsZ : 1);
+      }
+      const int nb = s_g.nb[s];
+      const bool none = s >= 4 && nb < 0;  // no halo plane: the word goes nowhere
+      const bool local = nb < 0 || nb == rank;
+      s_push[u] = local ? make_uint2((uint32_t)src | kLocal, (uint32_t)(none ? src : dst))
+                        : make_uint2((uint32_t)src, (uint32_t)(nb * 2 * P::n * hw + far));
+      s_pull[u] = local ? kLocal : (uint32_t)fill;
+    }
+    __syncthreads();
+    auto info = [&](int m) { return s_info[m * TH + tid]; };
+    auto count = [&](int m) { return (int)(s_info[m * TH + tid].x >> kCnt & 7u); };
+    auto cell = [&](int m) { return s_cell[m * TH + tid]; };
+
+    // After the chunks of this CTA are in buffers b0 (and b0 ^ 1): the boundary cells go into
+    // the neighbours' halos; every halo of this CTA is in place on return.  False after a
+    // timeout.
+    auto exchange = [&](int b0, int nchan) -> bool {
+      ++seq;
+      __syncthreads();
+#pragma unroll 1
+      for (int ch = 0; ch < nchan; ++ch) {
+        N* const D = (b0 ^ ch) ? D1 : D0;
+        unsigned long long* const far = s_g.halo + (size_t)((int)(seq & 1) * P::n + ch) * hw * NW;
+#pragma unroll 1
+        for (int u = tid; u < nu; u += TH) {
+          const uint2 e = s_push[u];
+          const auto c = ld_chunk(D + (e.x & 0xffffu));
+          if (e.x & kLocal) {
+            st_chunk(D + e.y, c.v);
+          } else {
+#pragma unroll
+            for (int k = 0; k < kRsZ * NW; k += 2)
+              put2(far + (size_t)e.y * NW + k, as_word(c.v[k / NW], k % NW), as_word(c.v[(k + 1) / NW], (k + 1) % NW), seq);
+          }
+        }
+#pragma unroll 1
+        for (int u = nu + tid; u < nu + nw; u += TH) {
+          const uint2 e = s_push[u];
+          const N c = D[e.x & 0xffffu];
+          if (e.x & kLocal) D[e.y] = c;
+          else if constexpr (NW == 1) put1(far + e.y, as_word(c, 0), seq);
+          else put2(far + (size_t)e.y * NW, as_word(c, 0), as_word(c, 1), seq);
+        }
+      }
+      if (G > 1) {
+#pragma unroll 1
+        for (int ch = 0; ch < nchan; ++ch)
+          if (!rs_receive<N, TH>((b0 ^ ch) ? D1 : D0, s_pull, nu, nw,
+                                 s_g.halo + (size_t)((rank * 2 + (int)(seq & 1)) * P::n + ch) * hw * NW, seq, a.ctl,
+                                 a.spin_limit))
+            s_ok = 0;
+      }
+      __syncthreads();
+      return s_ok;
+
+    };
+
+    T X[M][kRsZ];
+    N Q[M][kRsZ];
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+      for (int z = 0; z < kRsZ; ++z) {
+        X[m][z] = W::zero();
+        Q[m][z] = N(0);
+      }
+    for (int m_tau = 0; m_tau < a.n_tau; ++m_tau) {
+      const int ph = (a.scheme == TAU_BDF2 && m_tau > 0) ? 1 : 0;
+      const SmoothSpec& sp = md.sp[ph];
+      if constexpr (GR) {
+        for (int k = tid; k < 2 * bz; k += TH) {
+          if constexpr (sizeof(N) == 4) s_cz[k] = md.z.czf[ph][2 * z0 + k];
+          else s_cz[k] = (N)md.z.cz[ph][2 * z0 + k];
+        }
+      }
+      // ---- b from the previous pseudo-step's result (in registers; the first step loads
+      //      it); x, or the guess
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const int cnt = count(m);
+        if (!cnt) continue;
+        const int g = cell(m);
+#pragma unroll
+        for (int z = 0; z < kRsZ; ++z) {
+          if (z >= cnt) continue;
+          const int k = g + z * nxy;
+          const T xv = m_tau == 0 ? W::ld(s_g.x + k) : X[m][z];
+          s_g.b[k] = rhs_of<T>(a.scheme, m_tau, xv, s_g.xp ? s_g.xp + k : nullptr);
+          X[m][z] = m_tau == 0 && s_g.guess ? W::ld(s_g.guess + k) : xv;
+        }
+      }
+      int total = 0;
+      double bb = 0.0;
+      for (int round = 0; round < kMaxRounds; ++round) {
+        // ---- x published, its halos in place
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          const uint2 in = info(m);
+          if (!in.x) continue;
+#pragma unroll
+          for (int ch = 0; ch < P::n; ++ch) {
+            N v[kRsZ];
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z) v[z] = P::word(X[m][z], ch);
+            st_chunk((ch ? D1 : D0) + (in.x & 0xffffu), v);
+          }
+        }
+        if (!exchange(0, P::n)) return;
+        // ---- true residual (wide), its narrow copy to global memory, sums (each chunk's
+        //      in FP32, then compensated); the next chunk's b is loaded ahead
+        Sum sum[kQ] = {};
+        {
+          const T cf[3] = {coef_w<T>(sp, 0), coef_w<T>(sp, 1), coef_w<T>(sp, 2)};
+          T bn[kRsZ];
+          auto load_b = [&](int m) {
+            const int cnt = m < M ? count(m) : 0;
+            if (!cnt) return;
+            const T* const p = s_g.b + cell(m);
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z)
+              if (z < cnt) bn[z] = W::ld(p + z * nxy);
+          };
+          // one chunk; out(z, r) takes its residuals
+          auto chunk = [&](int m, auto&& out) {
+            const uint2 in = info(m);
+            const int o = (int)(in.x & 0xffffu), cnt = (int)(in.x >> kCnt & 7u);
+            [[maybe_unused]] const int kz = z0 + (int)(in.x >> kZc) * kRsZ;
+            T bv[kRsZ], c[kRsZ], l[kRsZ], r[kRsZ], fr[kRsZ], bk[kRsZ];
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z) bv[z] = bn[z];
+            load_b(m + 1);
+            P::chunk(D0, D1, o, c);
+            P::chunk(D0, D1, o - kRsZ, l);
+            P::chunk(D0, D1, o + kRsZ, r);
+            P::chunk(D0, D1, o - pr, fr);
+            P::chunk(D0, D1, o + pr, bk);
+            T below = P::one(D0, D1, (int)(in.y & 0xffffu));
+            const T top = P::one(D0, D1, (int)(in.y >> 16));
+            N sr2 = N(0), sr = N(0), sb2 = N(0);
+            [[maybe_unused]] N sw = N(0);
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z) {
+              if (z < cnt) {
+                const T above = z + 1 < kRsZ && z + 1 < cnt ? c[z + 1 < kRsZ ? z + 1 : z] : top;
+                N rn;
+                if constexpr (GR)
+                  rn = Resid<T>::eval_z(cf, md.z.cz[ph] + 2 * (kz + z), c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
+                else
+                  rn = Resid<T>::eval(cf, c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
+                out(z, rn);
+                sr2 += rn * rn;
+                sr += rn;
+                if constexpr (GR) sw += (N)md.z.w[kz + z] * rn;
+                if (round == 0) {
+                  const N b1 = W::narrow(bv[z]);
+                  sb2 += b1 * b1;
+                }
+              }
+              below = c[z];
+            }
+            sum[0].add(sr2);
+            sum[1].add(sr);
+            if (round == 0) sum[2].add(sb2);
+            if constexpr (GR) sum[3].add(sw);
+          };
+          load_b(0);
+          // rolled (x and q fill the registers): the residuals pass through global memory
+#pragma unroll 1
+          for (int m = 0; m < M && count(m); ++m) {
+            N* const rg = s_g.r + cell(m);
+            chunk(m, [&](int z, N rn) { rg[z * nxy] = rn; });
+          }
+        }
+        // ---- the group's sums: warp (a reduce-scatter of the four), CTA, then the CTAs in
+        //      rank order
+        ++rseq;
+        {
+          Sum s2[2];
+          const bool h4 = lane & 16, h3 = lane & 8;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) s2[q] = Sum::give(sum[q], sum[q + 2], h4, 16);
+          Sum t = Sum::give(s2[0], s2[1], h3, 8);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) t.join(o);
+          if ((lane & 7) == 0) s_red[wid][(h4 ? 2 : 0) + (h3 ? 1 : 0)] = t;
+        }
+        __syncthreads();
+        if (wid == 0) {
+          // lane: sum lane >> 3 of warps lane & 7, ...
+          Sum t = s_red[lane & 7][lane >> 3];
+          for (int r = (lane & 7) + 8; r < kWarps; r += 8) t.plus(s_red[r][lane >> 3]);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) t.join(o);
+          if ((lane & 7) == 0) s_tot[lane >> 3] = t.d();
+          __syncwarp();
+          if (G > 1 && lane < kQ) {
+            const double v = s_tot[lane];
+            put2(s_g.sums + (((size_t)(rseq & 1) * G + rank) * kQ + lane) * 2, as_word(v, 0), as_word(v, 1), rseq);
+          }
+        }
+        if (G > 1) {
+          bool ok = true;
+          for (int t = tid; t < G * kQ; t += TH) {
+            const unsigned long long* p = s_g.sums + ((size_t)(rseq & 1) * G * kQ + t) * 2;
+            Tag2 v;
+            v.load(p);
+            Spin spin;
+            while (!v.is(rseq) && ok) {
+              ok = spin.go(a.ctl, a.spin_limit);
+              v.load(p);
+            }
+            of_words(s_part[t / kQ][t % kQ], (uint32_t)v.a, (uint32_t)v.b);
+          }
+          if (!ok) s_ok = 0;
+          __syncthreads();
+          if (!s_ok) return;
+        }
+        // the first warp of every CTA sums and decides: every CTA takes the same decision
+        if (wid == 0) {
+          if (G > 1) {
+            const int q = lane >> 3;
+            double t = 0.0;
+            for (int r = lane & 7; r < G; r += 8) t += s_part[r][q];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if ((lane & 7) == 0) s_tot[q] = t;
+            __syncwarp();
+          }
+          if (lane == 0) {
+            const double rr = s_tot[0], sr = s_tot[1];
+            if (round == 0) bb = s_tot[2];
+            const int zero = !(bb > 0.0);
+            double shift, rrp;
+            if (GR) {
+              // the shift keeps sum(w x) = sum(w b); |r - s|^2 = |r|^2 - 2 s sum r + C s^2
+              shift = zero ? 0.0 : s_tot[3] * s_g.inv;
+              rrp = fmax(rr - 2.0 * shift * sr + (double)C * shift * shift, 0.0);
+            } else {
+              shift = zero ? 0.0 : sr * s_g.inv;
+              rrp = fmax(rr - sr * (sr * s_g.inv), 0.0);
+            }
+            int k = 0;
+            if (!zero && !(rrp <= a.rtol2 * bb)) {
+              // |r_k| <= 2 sig^k |r_0|: enough steps for the tolerance, or for the reduction
+              // the narrow word can deliver in one round (the next round checks the true
+              // residual, so FP32 logarithms do)
+              const float need = fmaxf(0.5f * sqrtf((float)(a.rtol2 * bb / rrp)), (float)W::kFloor);
+              k = sp.sig > 0.0 ? (int)ceilf(logf(need) / logf((float)sp.sig)) : 1;
+              if (k < 1) k = 1;
+              if (k > kMaxStepsRound) k = kMaxStepsRound;
+              if (total + k > a.max_iter) k = a.max_iter - total;
+              if (k <= 0) {
+                k = 0;
+                if (rank == 0) atomicCAS((int*)&a.ctl->cg_status, 0, SEDI_EDIVERGED);
+              }
+            }
+            s_k = k;
+            s_shift = shift;
+            s_zero = zero;
+          }
+        }
+        __syncthreads();
+        const int k = s_k, zero = s_zero;
+        const double shift = s_shift;
+        total += k;
+        const T sw = W::from_d(shift);
+        // x back from its published copy (so it holds no registers during the residual)
+#pragma unroll
+        for (int m = 0; m < M; ++m) P::chunk(D0, D1, (int)(info(m).x & 0xffffu), X[m]);
+        if (k == 0) {
+          // converged (or zero, or stopped): the projection shift
+#pragma unroll
+          for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z) {
+              if (zero) X[m][z] = W::zero();
+              else if (shift != 0.0) X[m][z] = W::add(X[m][z], sw);
+            }
+          break;
+        }
+        // ---- the shift, q = r - s, and the first direction d = q / theta
+        const N shn = (N)shift;
+        N inv_theta;
+        if constexpr (sizeof(N) == 4) inv_theta = sp.inv_theta_f;
+        else inv_theta = (N)(1.0 / sp.theta);
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          const uint2 in = info(m);
+          if (!in.x) continue;
+          const int cnt = (int)(in.x >> kCnt & 7u);
+          const N* const rg = s_g.r + cell(m);
+          N v[kRsZ];
+#pragma unroll
+          for (int z = 0; z < kRsZ; ++z) {
+            v[z] = N(0);
+            if (z >= cnt) continue;
+            Q[m][z] = rg[z * nxy] - shn;
+            v[z] = Q[m][z] * inv_theta;
+            X[m][z] = W::add(X[m][z], sw);
+          }
+          st_chunk(D0 + (in.x & 0xffffu), v);
+        }
+        if (!exchange(0, 1)) return;
+        // ---- Chebyshev steps
+        const N cfn[3] = {coef_w<N>(sp, 0), coef_w<N>(sp, 1), coef_w<N>(sp, 2)};
+#pragma unroll 1
+        for (int j = 1; j <= k; ++j) {
+          const N* const D = (j & 1) ? D0 : D1;
+          N* const Dn = (j & 1) ? D1 : D0;
+          N c1, c2;
+          if constexpr (sizeof(N) == 4) {
+            c1 = sp.chebf[0][j - 1];
+            c2 = sp.chebf[1][j - 1];
+          } else {
+            c1 = (N)sp.cheb[0][j - 1];
+            c2 = (N)sp.cheb[1][j - 1];
+          }
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            const uint2 in = info(m);
+            if (!in.x) continue;
+            const int o = (int)(in.x & 0xffffu);
+            const auto c = ld_chunk(D + o), l = ld_chunk(D + o - kRsZ), r = ld_chunk(D + o + kRsZ);
+            const auto fr = ld_chunk(D + o - pr), bk = ld_chunk(D + o + pr);
+            N below = D[in.y & 0xffffu], v[kRsZ];
+            const N top = D[in.y >> 16];
+            N up[kRsZ] = {c.v[1], c.v[2], c.v[3], top};
+            if (part) {  // the brick's last chunk ends before its fourth cell
+              const int cnt = (int)(in.x >> kCnt & 7u);
+              if (cnt == 1) up[0] = top;
+              if (cnt == 2) up[1] = top;
+              if (cnt == 3) up[2] = top;
+            }
+#pragma unroll
+            for (int z = 0; z < kRsZ; ++z) {
+              const N cur = c.v[z], above = up[z];
+              const N sx = (l.v[z] - cur) + (r.v[z] - cur);
+              const N sy = (fr.v[z] - cur) + (bk.v[z] - cur);
+              N lap = cfn[0] * sx + cfn[1] * sy;
+              if constexpr (GR) {
+                const N* const cz = s_cz + 2 * ((int)(in.x >> kZc) * kRsZ + z);
+                const N tm = cz[0] * (below - cur), tp = cz[1] * (above - cur);
+                lap = (lap + tm) + tp;
+              } else {
+                lap = lap + cfn[2] * ((below - cur) + (above - cur));
+              }
+              Q[m][z] = Q[m][z] - (cur - lap);
+              v[z] = c1 * cur + c2 * Q[m][z];
+              X[m][z] = W::add_n(X[m][z], cur);
+              below = cur;
+            }
+            if (j < k) st_chunk(Dn + o, v);
+          }
+          if (j < k && !exchange(j & 1, 1)) return;
+        }
+        __syncthreads();  // every reader of the directions is done before x is published
+      }
+      if (rank == 0 && tid == 0 && md.iters) atomicAdd(md.iters + f, total);
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int cnt = count(m);
+      if (!cnt) continue;
+      T* const xg = s_g.x + cell(m);
+#pragma unroll
+      for (int z = 0; z < kRsZ; ++z)
+        if (z < cnt) xg[z * nxy] = X[m][z];
+    }
+  }
+}
+
 __global__ void k_bar_reset(Ctl* ctl) {
   ctl->bar_count = 0u;
   ctl->bar_gen = 0u;
@@ -1072,11 +1886,19 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 int64_t smooth_units(int64_t C) { return (C + kThreads - 1) / kThreads; }
 
+// Room for the resident solver's tagged words behind the direction arrays: another such
+// array for meshes beyond a cluster, 4 MB for the small meshes of the FP64 form.
+static size_t rs_extra(int form, int64_t C) {
+  if (form == FORM_PLAIN) return 0;
+  if (C > (int64_t)kClMaxCta * kClCells) return align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4));
+  return form == FORM_FP64 ? (size_t)kSmoothTagBytes : 0;
+}
+
 size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme) {
   const size_t w = form == FORM_PLAIN ? 4 : 8;             // wide word
   const size_t n = form == FORM_FP64 ? 8 : 4;              // narrow word
   const size_t wide = align256((size_t)nf * C * w);        // b, and x^{m-1} for BDF2
-  return (scheme == TAU_BDF2 ? 2 : 1) * wide + 3 * align256((size_t)kMaxF * C * n) +
+  return (scheme == TAU_BDF2 ? 2 : 1) * wide + 3 * align256((size_t)kMaxF * C * n) + rs_extra(form, C) +
          align256((size_t)smooth_units(C) * kMaxF * kQ * 8) + 256;
 }
 
@@ -1087,7 +1909,7 @@ size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme) {
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf, void* work,
                   const DevState& st, int* iters_dev, double rtol, int max_iter, int n_tau,
                   int scheme, const double coef[3], const SmoothZ* z, cudaStream_t s,
-                  long long spin_limit) {
+                  long long spin_limit, bool averaging) {
   SmoothMesh m{};
   m.phi = phi;
   m.guess = guess;
@@ -1103,7 +1925,7 @@ int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, in
   if (z) m.z = *z;
   void* batch = (char*)work + align256(smooth_mesh_bytes(form, P.C, nf, scheme));
   return launch_smooth_batch(form, &m, 1, nf, batch, rtol, max_iter, n_tau, scheme, st.ctl,
-                             1 << 30, s, spin_limit);
+                             1 << 30, s, spin_limit, averaging);
 }
 
 size_t smooth_batch_bytes(int64_t B, int64_t U) {
@@ -1159,7 +1981,8 @@ static void smooth_mesh_layout(int form, int scheme, const SmoothMesh& in, Smoot
   m.q = p;
   m.d[0] = p + nar;
   m.d[1] = p + 2 * nar;
-  p += 3 * nar;
+  m.halo_bytes = (int64_t)(2 * nar + rs_extra(form, in.C));
+  p += 3 * nar + rs_extra(form, in.C);
   m.part = (double*)p;
   m.iters = in.iters;
   m.C = in.C;
@@ -1230,39 +2053,168 @@ void cluster_plan(int form, const SmoothMeshDev& m, int* csize, int* planes) {
   *planes = p;
 }
 
+// How the resident solver cuts a mesh into px x py x pz bricks (G CTAs), or G = 0 when no
+// cut fits.  The choice depends on the mesh, the form and the device alone, so a mesh is
+// smoothed with the same bits in any batch.
+struct RsPlan {
+  int G = 0, px = 0, py = 0, pz = 0, groups = 0;
+  int chunks = 0;             // of a thread
+  size_t smem = 0, halo = 0;  // dynamic shared memory; halo words of a CTA and channel
+};
+
+// Bytes of a CTA's tagged words: two parities of the sums and of the halo words (the
+// double-float form has two channels of 4-byte words, FP64 one of 8 bytes).
+size_t rs_tag_bytes(size_t halo) { return 2 * kQ * 16 + halo * 4 * 8; }
+
+// Fields of FP32 words that a thread's few chunks hold go to one CTA: no exchange at all,
+// and many meshes in one launch.
+bool rs_one_cta(int form, const SmoothMeshDev& m) {
+  return form == FORM_SPLIT &&
+         (int64_t)m.nc[0] * m.nc[1] * ((m.nc[2] + kRsZ - 1) / kRsZ) <= kRsThreads * kRsChunks;
+}
+
+RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
+  const size_t word = form == FORM_FP64 ? 8 : 4;
+  const int nx = m.nc[0], ny = m.nc[1], nz = m.nc[2];
+  const int T = kRsThreads, top = T * (word == 8 ? kRsChunks : kRsChunksBig);
+  RsPlan best;
+  double best_cost = 1e300;
+  auto consider = [&](int px, int py, int pz, int groups) {
+    if (px < 1 || px > nx || py > ny || pz > nz) return;
+    const int G = px * py * pz;
+    const int64_t bx = (nx + px - 1) / px, by = (ny + py - 1) / py, bz = (nz + pz - 1) / pz;
+    const int64_t nzc = (bz + kRsZ - 1) / kRsZ, nch = bx * by * nzc;
+    if (nch > top) return;
+    const bool zcut = pz > 1 || m.per[2];
+    const int64_t words = (nzc * (by + 2) * ((bx + 2) | 1) * kRsZ + (zcut ? 2 * bx * by : 0) + 3) / 4 * 4;
+    const int64_t nu = 2 * nzc * (bx + by) + (zcut ? 2 * bx * by : 0);
+    const size_t smem = (2 * (size_t)words + 2 * (size_t)nzc * kRsZ) * word + (size_t)nu * 12;
+    // a chunk's word holds 16 bits of index and 11 of its place along z
+    if (smem > kRsSmem || words > 0xffff || nzc > 2000) return;
+    const size_t halo = 2 * (size_t)(nzc * kRsZ * (bx + by) + (zcut ? bx * by : 0));
+    // time of a step, in microseconds, fitted to measured cuts of 128 x 64 x 128 and
+    // 256 x 128 x 64 meshes: 0.45 for every 512 chunks (FP64: by the cells, its pipe is
+    // the limit); an exchange's latency, its halo chunks and its plane words (tagged words
+    // cost most: they fill L2's write path)
+    const int chunks = (int)((nch + T - 1) / T);
+    const double units = 2.0 * (double)(nzc * (bx + by)), planes = zcut ? 2.0 * (double)(bx * by) : 0.0;
+    double t = word == 8 ? 0.006 * (double)(nch * kRsZ) : 0.45 * chunks;
+    if (G > 1) {
+      // every group's tagged sums and halo words live in the direction arrays of the
+      // mesh's scratch
+      if ((int64_t)rs_tag_bytes(halo) * groups * G > m.halo_bytes) return;
+      t += 1.5 + 0.0018 * units + 0.00015 * planes;
+    }
+    const double cost = t * ((7 + groups - 1) / groups);  // waves of the averaging's seven fields
+    if (cost < best_cost) {
+      best_cost = cost;
+      best.G = G;
+      best.px = px;
+      best.py = py;
+      best.pz = pz;
+      best.groups = groups;
+      best.chunks = chunks;
+      best.smem = smem;
+      best.halo = halo;
+    }
+  };
+  if (rs_one_cta(form, m)) {
+    consider(1, 1, 1, 1);
+    if (best.G) return best;
+  }
+  // for every number of groups at once, the largest groups
+  for (int g = 1; g <= 7; ++g) {
+    const int gmax = nsm / g < kRsMaxGroup ? nsm / g : kRsMaxGroup;
+    for (int pz = 1; pz <= 40 && pz <= gmax; ++pz)
+      for (int py = 1; py * pz <= gmax; ++py) consider(gmax / (py * pz), py, pz, g);
+  }
+  return best;
+}
+
+// The fields of one mesh over the groups of a cooperative launch (every CTA resident, one
+// per SM), or the fields of many meshes of one CTA each, an ordinary launch.
+template <class T, bool GR>
+int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m, int nsm, cudaStream_t s) {
+  auto* kern = k_smooth_rs<T, GR, kRsChunks>;
+  if constexpr (!std::is_same<T, double>::value)
+    if (pl.chunks > kRsChunks) kern = k_smooth_rs<T, GR, kRsChunksBig>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsSmem) != cudaSuccess)
+    return -3;
+  if (pl.G == 1) {
+    const int64_t items = (int64_t)a.B * a.nf;
+    kern<<<(unsigned)(items < nsm ? items : nsm), kRsThreads, pl.smem, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  }
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRsThreads, pl.smem) != cudaSuccess) return -3;
+  const int groups = pl.groups < a.nf ? pl.groups : a.nf;
+  if ((int64_t)per_sm * nsm < (int64_t)groups * pl.G) return -3;
+  // no tagged word of an earlier launch may pass for this one's: exchanges count from 1
+  const size_t bytes = rs_tag_bytes(pl.halo) * groups * pl.G;
+  if (cudaMemsetAsync(m.d[0], 0, bytes, s) != cudaSuccess) return -3;
+  SmoothBatchDev args = a;
+  void* p[] = {&args};
+  return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)(groups * pl.G)), dim3(kRsThreads), p, pl.smem, s) ==
+                 cudaSuccess
+             ? 0
+             : -3;
+}
+
 }  // namespace
 
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit) {
+                        int max_blocks, cudaStream_t s, long long spin_limit, bool averaging) {
   if (B < 1 || B > kMaxBeds || nf < 1 || nf > kMaxF || (scheme != TAU_EULER && scheme != TAU_BDF2))
     return -1;
   // every mesh of a batch is graded or none is (one kernel instantiation per launch)
   const bool gr = meshes[0].z.cz[0] != nullptr;
   for (int b = 1; b < B; ++b)
     if ((meshes[b].z.cz[0] != nullptr) != gr) return -1;
-  // meshes that fit the cluster solver take it; the rest take the grid solver.  The
-  // choice depends on the mesh alone, so a bed smooths the same way in any batch.
-  std::vector<SmoothMeshDev> mg, mc;
-  int64_t U = 0;
-  for (int b = 0; b < B; ++b) {
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (nsm > max_blocks) nsm = max_blocks;
+  // FP32 words: meshes beyond one CTA that fit a cluster's shared memory take the cluster
+  // solver (one launch for every mesh of a cluster size).  Fields that fit one CTA and
+  // meshes that fit the whole chip take the resident solver, the rest the streaming grid
+  // solver.  The averaging of the FP32-force forms keeps the cluster and streaming solvers:
+  // the resident one differs from them in the last bits (~1e-11, far inside the tolerance),
+  // and an averaged solid fraction that rounds to another FP32 word changes the drag and
+  // with it a trajectory.  The plain form keeps them as the baseline.  The choice
+  // depends on the mesh alone, so a bed smooths the same way in any batch.
+  struct Item {
     SmoothMeshDev m;
-    smooth_mesh_layout(form, scheme, meshes[b], &m);
-    int cs, pl;
-    cluster_plan(form, m, &cs, &pl);
+    RsPlan pl;
+  };
+  std::vector<SmoothMeshDev> mg, mc;
+  std::vector<Item> mr;
+  for (int b = 0; b < B; ++b) {
+    Item it;
+    smooth_mesh_layout(form, scheme, meshes[b], &it.m);
+    const bool rs = form == FORM_FP64 || (form == FORM_SPLIT && !averaging);
+    int cs = 0, planes = 0;
+    if (!rs || !rs_one_cta(form, it.m)) cluster_plan(form, it.m, &cs, &planes);
+    if (rs && cs == 0) it.pl = rs_plan(form, it.m, nsm);
     if (cs > 0) {
-      m.cl_size = cs;
-      m.cl_planes = pl;
-      mc.push_back(m);
+      it.m.cl_size = cs;
+      it.m.cl_planes = planes;
+      mc.push_back(it.m);
+    } else if (it.pl.G > 0) {
+      it.m.rs_G = it.pl.G;
+      it.m.rs_px = it.pl.px;
+      it.m.rs_py = it.pl.py;
+      it.m.rs_pz = it.pl.pz;
+      mr.push_back(it);
     } else {
-      m.u0 = U;
-      U += m.nu;
-      mg.push_back(m);
+      mg.push_back(it.m);
     }
   }
-  // cluster meshes grouped by cluster size (one launch per size)
+  // cluster meshes grouped by cluster size (one launch per size), resident ones with the
+  // meshes of one CTA first (one launch for all)
   std::stable_sort(mc.begin(), mc.end(),
                    [](const SmoothMeshDev& x, const SmoothMeshDev& y) { return x.cl_size < y.cl_size; });
+  std::stable_sort(mr.begin(), mr.end(), [](const Item& x, const Item& y) { return (x.pl.G == 1) > (y.pl.G == 1); });
   char* p = (char*)batch_work;
   SmoothBatchDev a{};
   a.nf = nf;
@@ -1277,8 +2229,10 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
   SmoothMeshDev* tab_c = (SmoothMeshDev*)p;
   p += align256((size_t)B * sizeof(SmoothMeshDev));
   int rc = 0;
-  if (!mc.empty()) {
-    if (cudaMemcpyAsync(tab_c, mc.data(), mc.size() * sizeof(SmoothMeshDev), cudaMemcpyHostToDevice, s) != cudaSuccess)
+  if (!mc.empty() || !mr.empty()) {
+    std::vector<SmoothMeshDev> tab(mc);
+    for (const auto& it : mr) tab.push_back(it.m);
+    if (cudaMemcpyAsync(tab_c, tab.data(), tab.size() * sizeof(SmoothMeshDev), cudaMemcpyHostToDevice, s) != cudaSuccess)
       return -3;
     for (size_t i0 = 0; i0 < mc.size();) {
       size_t i1 = i0;
@@ -1293,21 +2247,47 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
         rc = form == FORM_SPLIT ? launch_cluster<dd, false>(c, mc[i0].cl_size, s)
                                 : launch_cluster<float, false>(c, mc[i0].cl_size, s);
       if (rc) {
-        // a device without this cluster shape: these meshes take the grid solver
+        // a device without this cluster shape: these meshes take the streaming solver
         cudaGetLastError();
         for (size_t i = i0; i < i1; ++i) {
           SmoothMeshDev m = mc[i];
           m.cl_size = m.cl_planes = 0;
-          m.u0 = U;
-          U += m.nu;
           mg.push_back(m);
         }
         rc = 0;
       }
       i0 = i1;
     }
+    for (size_t i0 = 0; i0 < mr.size();) {
+      // every mesh of one CTA in one launch, the larger ones one by one
+      size_t i1 = i0 + 1;
+      RsPlan pl = mr[i0].pl;
+      for (; pl.G == 1 && i1 < mr.size() && mr[i1].pl.G == 1; ++i1) {
+        pl.smem = std::max(pl.smem, mr[i1].pl.smem);
+        pl.chunks = std::max(pl.chunks, mr[i1].pl.chunks);
+      }
+      SmoothBatchDev c = a;
+      c.mesh = tab_c + mc.size() + i0;
+      c.B = (int32_t)(i1 - i0);
+      c.rs_G = pl.G;
+      if (form == FORM_SPLIT)
+        rc = gr ? launch_rs<dd, true>(c, pl, mr[i0].m, nsm, s) : launch_rs<dd, false>(c, pl, mr[i0].m, nsm, s);
+      else
+        rc = gr ? launch_rs<double, true>(c, pl, mr[i0].m, nsm, s) : launch_rs<double, false>(c, pl, mr[i0].m, nsm, s);
+      if (rc) {
+        cudaGetLastError();
+        for (size_t i = i0; i < i1; ++i) mg.push_back(mr[i].m);
+        rc = 0;
+      }
+      i0 = i1;
+    }
   }
   if (!mg.empty()) {
+    int64_t U = 0;
+    for (auto& m : mg) {
+      m.u0 = U;
+      U += m.nu;
+    }
     std::vector<int32_t> ub(U);
     for (size_t b = 0; b < mg.size(); ++b)
       for (int64_t u = 0; u < mg[b].nu; ++u) ub[mg[b].u0 + u] = (int32_t)b;
