@@ -46,3 +46,26 @@ def test_forward_and_gradient_on_ragged_meshes(ncell, periodic):
     loss_ref, grad_ref = orc.cnn_loss_grad(p, x, t, ncell, periodic)
     assert abs(loss - loss_ref) <= 2e-2 * loss_ref
     assert np.linalg.norm(grad - grad_ref) < 5e-2 * np.linalg.norm(grad_ref)
+
+
+@pytest.mark.parametrize("ncell,periodic", [
+    ((8, 8, 4), (1, 1, 0)), ((9, 8, 5), (0, 1, 1)), ((7, 9, 3), (1, 0, 1)), ((16, 4, 8), (0, 0, 0)),
+    ((1, 1, 1), (1, 1, 1)), ((2, 33, 9), (1, 1, 1)), ((41, 37, 30), (1, 1, 0))])
+def test_exact_sums_at_tile_edges(ncell, periodic):
+    """Fields of -1, 0, 1 and sparse weights of the same: every activation is a whole number
+    below 256, a bfloat16 word, so the output is exact, and the gradients differ from the FP64
+    ones by their FP32 sums alone: a random walk over 27 x 32 products and the voxels,
+    sqrt(5e4) 2^-25 = 7e-6 at the largest mesh if nothing were summed in parts."""
+    hi = tuple(1e-3 * n for n in ncell)
+    g = sedi.Sedi(default_params(hi=hi, ncell=ncell, periodic=periodic, wall_lo=(0, 0, 0), wall_hi=(0, 0, 0)))
+    rng = np.random.default_rng(31)
+    p = np.concatenate([rng.integers(-1, 2, n) * (rng.random(n) < q) for n, q in (
+        (3456, .2), (32, 1), (27648, .04), (32, 1), (3456, .2), (4, 1))]).astype(np.float64)
+    g.cnn_set_params(p)
+    C = int(np.prod(ncell))
+    x, t = rng.integers(-1, 2, (4, C)).astype(float), rng.integers(-9, 10, (4, C)).astype(float)
+    np.testing.assert_array_equal(g.cnn_forward(x), orc.cnn_forward(p, x, ncell, periodic, round_bf16=True))
+    loss, grad = g.cnn_loss_grad(x, t)
+    loss_ref, grad_ref = orc.cnn_loss_grad(p, x, t, ncell, periodic)
+    assert abs(loss - loss_ref) <= 1e-12 * loss_ref
+    assert np.linalg.norm(grad - grad_ref) <= 7e-6 * np.linalg.norm(grad_ref)
