@@ -1344,15 +1344,14 @@ static int deposit_dev(sedi_handle* h) {
   return 0;
 }
 
-static int smooth_dev(sedi_handle* h, int nf, const void* guess, bool averaging, int n_tau = -1,
-                      bool zero_iters = true) {
+static int smooth_dev(sedi_handle* h, int nf, const void* guess, int n_tau = -1, bool zero_iters = true) {
   if (zero_iters) CK(cudaMemsetAsync(h->iters_dev, 0, 4 * 8, h->stream));
   // FP32 words cannot reach a relative residual much below 1e-6
   const double rtol = h->form == FORM_PLAIN ? std::max(h->prm.cg_rtol, 2e-6) : h->prm.cg_rtol;
   int rc = launch_smooth(h->form, h->P, h->phi, guess, nf, h->work, h->st, h->iters_dev,
                          rtol, h->prm.cg_max_iter, n_tau > 0 ? n_tau : h->prm.n_tau,
                          h->prm.tau_scheme, h->coef, h->P.graded ? &h->zs : nullptr,
-                         h->stream, h->barrier_spins, averaging);
+                         h->stream, h->barrier_spins);
   if (rc) return fail(h, SEDI_ECUDA, "cooperative launch of the smoother failed: %s", cudaGetErrorString(cudaGetLastError()));
   return 0;
 }
@@ -1388,7 +1387,7 @@ static int smooth_warm(sedi_handle* h) {
     float* y = nullptr;
     cnn_forward(h->P, h->cnn_master, h->cnn_work, &y, h->stream);
     cnn_guess(h->form, h->phi, y, scale, h->qfix, C, h->stream);
-    if ((rc = smooth_dev(h, 7, h->qfix, true, 1, false))) return rc;
+    if ((rc = smooth_dev(h, 7, h->qfix, 1, false))) return rc;
   }
   return 0;
 }
@@ -1839,7 +1838,7 @@ static int ens_average(sedi_handle* h) {
   const double rtol = h->form == FORM_PLAIN ? std::max(h->prm.cg_rtol, 2e-6) : h->prm.cg_rtol;
   if (launch_smooth_batch(h->form, m.data(), B, 7, h->ens_smooth, rtol, h->prm.cg_max_iter,
                           h->prm.n_tau, h->prm.tau_scheme, h->st.ctl, 1 << 30, h->stream,
-                          h->barrier_spins, true))
+                          h->barrier_spins))
     return fail(h, SEDI_ECUDA, "cooperative launch of the batched smoother failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
   launch_eps_out_ens(h->form, h->ens, h->stream);
@@ -1938,7 +1937,7 @@ static int average_from_fixed(sedi_handle* h, double* eps, double* Us, double* F
   if (h->prm.profile) CK(cudaEventRecord(h->avg_ev[1], h->stream));
   if (h->prm.use_cnn_guess && h->cnn_set) {
     if ((rc = smooth_warm(h))) return rc;
-  } else if ((rc = smooth_dev(h, 7, nullptr, true))) {
+  } else if ((rc = smooth_dev(h, 7, nullptr))) {
     return rc;
   }
   if (h->prm.profile) {
@@ -2132,7 +2131,7 @@ int sedi_smooth(sedi_handle* h, int32_t bed, int32_t nf, const double* in, doubl
     if (nf * C * wb > (size_t)8 * 7 * C) return fail(h, SEDI_EINVAL, "guess supports at most 7 fields");
     launch_phi_from_double(h->form, h->dstage + n, gdev, n, h->stream);
   }
-  if ((rc = smooth_dev(h, nf, gdev, false))) return rc;
+  if ((rc = smooth_dev(h, nf, gdev))) return rc;
   launch_phi_convert(h->form, h->phi, h->dstage, n, 1, h->stream);
   if ((rc = copy_out(h, out, h->dstage, 8 * n, mem))) return rc;
   int it[8] = {0};

@@ -1041,8 +1041,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
 // CTA (ix, iy, iz) of the group holds a brick of bx x by x bz cells.
 // x (wide) and the recursive residual q live in registers (a thread owns chunks of
 // kRsZ cells along z), the direction d in shared memory, double-buffered, with halos.
-// Same iteration, and the same FP32 recursion per cell, as the grid solver above: only
-// the association of the sums of a round and the low bits of the true residual differ.
+// Same iteration as the solvers above, operation for operation; in FP32 words the sums of a
+// round are theirs too (rs_sums), so are all bits of a result.
 // Halos between CTAs go through global memory (they stay in L2) as 8-byte words of a value
 // and the exchange's number, so a receiver polls the data itself: no fence, no flag and no
 // barrier between a store and its use.  A round's sums travel the same way.  Every wait is
@@ -1059,12 +1059,12 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
 // for four, so z is cut last.
 //
 // What bounds it: the exchange and the issue of a step.  On 128 x 64 x 128 a step takes
-// 7.3 us for 6,900 cells a CTA, of which the FP32 pipe accounts for 0.9 us (29 operations
-// a cell at 128 a clock and SM; packed f32x2 instructions run at the same operation rate),
-// one way between SMs through L2 for 0.8 us.
+// 8 us for 6,900 cells a CTA (rounds included), of which the FP32 pipe accounts for 0.9 us
+// (29 operations a cell at 128 a clock and SM; packed f32x2 instructions run at the same
+// operation rate), one way between SMs through L2 for 0.8 us.
 // Seven fields of random values, microseconds a call, streaming grid solver -> here:
-// 128 x 64 x 128 9,790 -> 4,960, 256 x 128 x 64 10,190 -> 5,590, 96 x 96 x 24
-// 2,020 -> 980; 10 x 10 x 20 in one CTA 440 -> 200; FP64 19 x 15 x 31 4,400 -> 710 (the
+// 128 x 64 x 128 9,760 -> 5,990, 256 x 128 x 64 10,190 -> 7,360, 96 x 96 x 24
+// 2,030 -> 1,140; 10 x 10 x 20 in one CTA 440 -> 250; FP64 19 x 15 x 31 4,390 -> 740 (the
 // streaming solver ran it on 35 blocks).
 constexpr int kRsZ = 4;              // cells of a chunk
 constexpr int kRsMaxGroup = 160;     // CTAs of a group at most
@@ -1075,33 +1075,6 @@ constexpr size_t kRsSmem = 176 * 1024;  // dynamic shared memory of a CTA at mos
 constexpr int kRsThreads = 512;
 constexpr int kRsChunks = 4;         // where they do, and in FP64
 constexpr int kRsChunksBig = 7;      // larger meshes
-
-// Sums of a round: FP32 residuals add up compensated (double-float), so a thread may sum
-// many cells, and a warp stays off the narrow FP64 pipe.
-struct SumF {
-  dd v;
-  __device__ void add(float x) { v = dd_add_f(v, x); }
-  __device__ void join(int o) {
-    v = dd_add(v, dd{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
-  }
-  __device__ void plus(const SumF& o) { v = dd_add(v, o.v); }
-  // a reduce-scatter step: keep one of two sums (b where up), added to the partner's
-  __device__ static SumF give(const SumF& a, const SumF& b, bool up, int o) {
-    const dd keep = up ? b.v : a.v, out = up ? a.v : b.v;
-    return SumF{dd_add(keep, dd{__shfl_xor_sync(0xffffffffu, out.hi, o), __shfl_xor_sync(0xffffffffu, out.lo, o)})};
-  }
-  __device__ double d() const { return dd_to_double(v); }
-};
-struct SumD {
-  double v;
-  __device__ void add(double x) { v += x; }
-  __device__ void join(int o) { v += __shfl_xor_sync(0xffffffffu, v, o); }
-  __device__ void plus(const SumD& o) { v += o.v; }
-  __device__ static SumD give(const SumD& a, const SumD& b, bool up, int o) {
-    return SumD{(up ? b.v : a.v) + __shfl_xor_sync(0xffffffffu, up ? a.v : b.v, o)};
-  }
-  __device__ double d() const { return v; }
-};
 
 // The four cells of a chunk as loaded from a direction buffer.
 struct C4f {
@@ -1165,50 +1138,14 @@ struct Resid {
                           W::mul(cf[2], pair(dn, up, c)));
     return W::narrow(W::subq(b, W::subq(c, lap)));
   }
-  __device__ static N eval_z(const T (&cf)[3], const double* cz, T c, T l, T r, T f, T k, T dn, T up, T b) {
+  // zz: the z faces' terms are added to each other first (the cluster solver's order)
+  __device__ static N eval_z(const T (&cf)[3], const double* cz, bool zz, T c, T l, T r, T f, T k, T dn, T up, T b) {
     T lap = W::addq(W::mul(cf[0], pair(l, r, c)), W::mul(cf[1], pair(f, k, c)));
-    lap = W::addq(lap, W::mul(W::from_d(cz[0]), W::subq(dn, c)));
-    lap = W::addq(lap, W::mul(W::from_d(cz[1]), W::subq(up, c)));
+    const T tm = W::mul(W::from_d(cz[0]), W::subq(dn, c)), tp = W::mul(W::from_d(cz[1]), W::subq(up, c));
+    lap = zz ? W::addq(lap, W::addq(tm, tp)) : W::addq(W::addq(lap, tm), tp);
     return W::narrow(W::subq(b, W::subq(c, lap)));
   }
 };
-// Double-float: the high words go through error-free sums and products, every error and
-// low word is collected in one FP32 sum, and nothing is renormalised on the way (98
-// operations a cell instead of 165; its error, a few 2^-47 of |x|, is below that of the
-// renormalising additions, 2^-44).
-template <>
-struct Resid<dd> {
-  // cf * ((m - c) + (p - c)) as an unnormalised pair
-  __device__ static dd axis(dd cf, dd m, dd p, dd c) {
-    const dd s = two_sum(m.hi, p.hi);
-    const dd t = two_sum(s.hi, -2.0f * c.hi);
-    const float lo = (s.lo + t.lo) + ((m.lo + p.lo) - 2.0f * c.lo);
-    const dd q = two_prod(cf.hi, t.hi);
-    return dd{q.hi, __fmaf_rn(cf.hi, lo, __fmaf_rn(cf.lo, t.hi, q.lo))};
-  }
-  __device__ static dd face(dd cf, dd m, dd c) {
-    const dd t = two_sum(m.hi, -c.hi);
-    const dd q = two_prod(cf.hi, t.hi);
-    return dd{q.hi, __fmaf_rn(cf.hi, t.lo + (m.lo - c.lo), __fmaf_rn(cf.lo, t.hi, q.lo))};
-  }
-  __device__ static dd plus(dd a, dd b) {  // unnormalised
-    const dd s = two_sum(a.hi, b.hi);
-    return dd{s.hi, s.lo + (a.lo + b.lo)};
-  }
-  __device__ static float eval(const dd (&cf)[3], dd c, dd l, dd r, dd f, dd k, dd dn, dd up, dd b) {
-    const dd lap = plus(plus(axis(cf[0], l, r, c), axis(cf[1], f, k, c)), axis(cf[2], dn, up, c));
-    const dd v = plus(plus(b, dd{-c.hi, -c.lo}), lap);
-    return __fadd_rn(v.hi, v.lo);
-  }
-  __device__ static float eval_z(const dd (&cf)[3], const double* cz, dd c, dd l, dd r, dd f, dd k, dd dn, dd up,
-                                 dd b) {
-    const dd xy = plus(axis(cf[0], l, r, c), axis(cf[1], f, k, c));
-    const dd zz = plus(face(dd_from_double(cz[0]), dn, c), face(dd_from_double(cz[1]), up, c));
-    const dd v = plus(plus(b, dd{-c.hi, -c.lo}), plus(xy, zz));
-    return __fadd_rn(v.hi, v.lo);
-  }
-};
-
 // Words that carry their own arrival: each 8-byte word of global memory holds 32 bits of
 // data and the number of the exchange that wrote it.  A 64-bit access is indivisible, so
 // a reader that finds the number has the data, with no fence between them.
@@ -1329,12 +1266,257 @@ __device__ __noinline__ bool rs_receive(N* D, const uint32_t* pull, int nu, int 
   return ok;
 }
 
+// A group's tagged words of the sums: a flag a CTA (its residuals are in place), then the
+// pieces below, each for two parities.
+constexpr int kRsPieces = kThreads;
+static_assert(kClMaxCta <= kRsPieces && kThreads == 256, "");
+__host__ __device__ constexpr size_t rs_sum_words(int G) { return 2 * ((size_t)G + 2 * kRsPieces * kQ); }
+
+// The sums of a round in FP32 words, in the order of the solver that takes this mesh
+// otherwise, so the choice of solver changes no bit of a result (an averaged solid
+// fraction that rounds to another FP32 word would change the drag and a trajectory with it).
+// A piece is what that solver adds in FP64 last: a CTA of its cluster (thread t of 1,024
+// adds columns t, t + 1,024, ..., a warp its threads, the CTA its 32 warps), or for the
+// streaming solver thread t of 256 that adds units t, t + 256, ... of 256 cells.
+// Piece p is formed by CTA p % G from the residuals in global memory and goes to
+// every CTA as tagged words.  This costs two exchanges and a read of the residuals from L2
+// a round: 1,000 of the 5,990 us of seven 128 x 64 x 128 fields, twelve rounds each.
+// ONE: a group of one CTA, its residuals in shared memory.
+template <class T, bool GR, bool ONE>
+__device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, const T* b, bool first, int G, int rank,
+                                     float* sl, unsigned long long* words, uint32_t seq, double* tot, int* s_ok,
+                                     Ctl* ctl, long long spin_limit) {
+  using W = Wide<T>;
+  constexpr int TH = kRsThreads, kWarps = TH / 32, kRanks = 10, kUnits = 40;  // 5,120 bytes of sl
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nxy = md.nc[0] * md.nc[1];
+  const int64_t C = md.C;
+  unsigned long long* const flags = words + (size_t)(seq & 1) * G;
+  unsigned long long* const pieces = words + 2 * (size_t)G + (size_t)(seq & 1) * 2 * kRsPieces * kQ;
+  __syncthreads();
+  if (!ONE) {
+    if (tid == 0) {
+      __threadfence();
+      put1(flags + rank, 0u, seq);
+    }
+    if (tid < G) {
+      Spin spin;
+      while ((uint32_t)(get1(flags + tid) >> 32) != seq)
+        if (!spin.go(ctl, spin_limit)) {
+          *s_ok = 0;
+          break;
+        }
+      __threadfence();
+    }
+    __syncthreads();
+    if (!*s_ok) return false;
+  }
+  auto put_piece = [&](int p, int q, double v) {
+    put2(pieces + ((size_t)p * kQ + q) * 2, as_word(v, 0), as_word(v, 1), seq);
+  };
+  bool ok = true;
+  auto get_piece = [&](int p, int q) {
+    const unsigned long long* const at = pieces + ((size_t)p * kQ + q) * 2;
+    Tag2 v;
+    v.load(at);
+    Spin spin;
+    while (!v.is(seq) && ok) {
+      ok = spin.go(ctl, spin_limit);
+      v.load(at);
+    }
+    double d;
+    of_words(d, (uint32_t)v.a, (uint32_t)v.b);
+    return d;
+  };
+  // warp sums of four values, a butterfly from 16 down for each: q0 and q2 in the lower
+  // half of the lanes, q1 and q3 in the upper
+  auto warp_sums = [&](float (&v)[kQ], float* to, int stride) {
+    const bool up = lane & 16;
+    float a = up ? v[1] : v[0], c = up ? v[3] : v[2];
+    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+    if (first || GR) c += __shfl_xor_sync(0xffffffffu, up ? v[2] : v[3], 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (first || GR) c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    if ((lane & 15) == 0) {
+      to[(up ? 1 : 0) * stride] = a;
+      to[(up ? 3 : 2) * stride] = c;
+    }
+  };
+  // warp sums of the 8 warps of a unit, two values each: the same butterflies as a
+  // reduce-scatter, a lane keeps half of its sums at every step
+  auto unit_warps = [&](float (&v)[2][8], float* to) {
+    float a[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      const bool up = lane & 16;
+      a[w] = (up ? v[1][w] : v[0][w]) + __shfl_xor_sync(0xffffffffu, up ? v[0][w] : v[1][w], 16);
+    }
+#pragma unroll
+    for (int o = 8; o > 1; o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int w = 0; w < o / 2; ++w)
+        a[w] = (up ? a[w + o / 2] : a[w]) + __shfl_xor_sync(0xffffffffu, up ? a[w] : a[w + o / 2], o);
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    if (!(lane & 1)) to[lane >> 1] = a[0];  // [value][warp]
+  };
+  auto load = [&](int64_t c) {
+    if constexpr (ONE) return r[c];
+    else return __ldcg(r + c);
+  };
+  if (md.cl_size > 0) {
+    const int cs = md.cl_size, P = md.cl_planes;
+    if (tid < kQ && ONE) tot[tid] = 0.0;
+    for (int r0 = rank; r0 < cs; r0 += kRanks * G) {
+      for (int i = 0; i < kRanks && r0 + i * G < cs; ++i) {
+        const int z0 = (r0 + i * G) * P, z1 = z0 + P < md.nc[2] ? z0 + P : md.nc[2];
+#pragma unroll 1
+        for (int t = tid; t < kClThreads; t += TH) {
+          float v[kQ] = {0.0f, 0.0f, 0.0f, 0.0f};
+          for (int s = t; s < nxy; s += kClThreads) {
+            constexpr int kAhead = 8;  // planes whose loads are under way together
+            for (int za = z0; za < z1; za += kAhead) {
+              float rn[kAhead];
+              T bv[kAhead];
+#pragma unroll
+              for (int k = 0; k < kAhead; ++k) {
+                const int64_t c = (int64_t)(za + k) * nxy + s;
+                rn[k] = za + k < z1 ? load(c) : 0.0f;
+                bv[k] = W::zero();
+                if (first) bv[k] = za + k < z1 ? W::ld(b + c) : W::zero();
+              }
+#pragma unroll
+              for (int k = 0; k < kAhead; ++k) {
+                if (za + k >= z1) continue;
+                v[0] += rn[k] * rn[k];
+                v[1] += rn[k];
+                if constexpr (GR) v[3] += (float)md.z.w[za + k] * rn[k];
+                const float bn = W::narrow(bv[k]);
+                v[2] += bn * bn;
+              }
+            }
+          }
+          warp_sums(v, sl + (i * 32 + (t >> 5)) * kQ, 1);
+        }
+      }
+      __syncthreads();
+      const int q = tid % kQ;
+      for (int i = ONE ? 0 : tid / kQ; i < kRanks && r0 + i * G < cs && tid < (ONE ? kQ : kRanks * kQ); ++i) {
+        double t = 0.0;
+        for (int w = 0; w < 32; ++w) t += (double)sl[(i * 32 + w) * kQ + q];
+        if (ONE) {
+          tot[q] += t;
+        } else {
+          put_piece(r0 + i * G, q, t);
+          break;
+        }
+      }
+      __syncthreads();
+    }
+    if (!ONE) {
+      double* const part = (double*)sl;
+      for (int k = tid; k < cs * kQ; k += TH) part[k] = get_piece(k / kQ, k % kQ);
+      if (!ok) *s_ok = 0;
+      __syncthreads();
+      if (tid < kQ) {
+        double t = 0.0;
+        for (int k = 0; k < cs; ++k) t += part[k * kQ + tid];
+        tot[tid] = t;
+      }
+    }
+  } else {
+    const int nu = (int)md.nu, np = nu < kRsPieces ? nu : kRsPieces;
+    const int mine = rank < np ? (np - rank + G - 1) / G : 0;  // this CTA's pieces rank, rank + G, ...
+    const int all = mine * ((nu + kRsPieces - 1) / kRsPieces);
+    double acc = 0.0;  // of piece tid / kQ of them (128 at most), sum tid % kQ
+    for (int i0 = 0; i0 < all; i0 += kUnits) {  // units in order for every piece
+      const int n = all - i0 < kUnits ? all - i0 : kUnits;
+#pragma unroll 1
+      for (int s = wid; s < n; s += kWarps) {  // a warp takes the 8 warps of a unit
+        const int i = i0 + s, u = rank + i % mine * G + i / mine * kRsPieces;
+        const int64_t c0 = (int64_t)u * kThreads + lane;
+        float rn[8], v[2][8];
+        T bv[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {  // every load before the first use
+          const int64_t c = c0 + w * 32;
+          const bool in = u < nu && c < C;
+          rn[w] = in ? load(c) : 0.0f;
+          bv[w] = W::zero();
+          if (first) bv[w] = in ? W::ld(b + c) : W::zero();
+        }
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+          v[0][w] = rn[w] * rn[w];
+          v[1][w] = rn[w];
+        }
+        unit_warps(v, sl + s * (8 * kQ));
+        if (GR || first) {
+#pragma unroll
+          for (int w = 0; w < 8; ++w) {
+            const float bn = W::narrow(bv[w]);
+            v[0][w] = bn * bn;
+            v[1][w] = 0.0f;
+            if constexpr (GR) {
+              const int c = (int)c0 + w * 32;
+              if (u < nu && c < C) v[1][w] = (float)md.z.w[c / nxy] * rn[w];
+            }
+          }
+          unit_warps(v, sl + s * (8 * kQ) + 16);
+        }
+      }
+      __syncthreads();
+      if (tid < n * kQ && (GR || first || tid % kQ < 2)) {  // a unit's sum, in the place of its warps'
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += (double)sl[tid * 8 + w];
+        ((double*)sl)[tid * 4] = t;
+      }
+      __syncthreads();
+      if (tid < mine * kQ) {
+        const int j = tid / kQ, q = tid % kQ;
+        for (int k = ((j - i0) % mine + mine) % mine; k < n; k += mine)
+          if (rank + j * G + (i0 + k) / mine * kRsPieces < nu) acc += ((double*)sl)[(k * kQ + q) * 4];
+      }
+      __syncthreads();
+    }
+    double* const own = (double*)sl;       // one CTA: the pieces
+    double* const ws = (double*)sl + 600;  // sums of 32 pieces
+    if (tid < mine * kQ) {
+      if (!ONE) put_piece(rank + tid / kQ * G, tid % kQ, acc);
+      else own[tid] = acc;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = wid; k < 8 * kQ; k += kWarps) {
+      const int p = k / kQ * 32 + lane, q = k % kQ;
+      double v = p < np ? (!ONE ? get_piece(p, q) : own[p * kQ + q]) : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) ws[k] = v;
+    }
+    if (!ok) *s_ok = 0;
+    __syncthreads();
+    if (tid < kQ) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += ws[w * kQ + tid];
+      tot[tid] = t;
+    }
+  }
+  __syncthreads();
+  return *s_ok;
+}
+
 template <class T, bool GR, int M>
 __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
   using W = Wide<T>;
   using N = typename W::N;
   using P = Pub<T>;
-  using Sum = typename std::conditional<sizeof(N) == 8, SumD, SumF>::type;
+  constexpr bool kOrder = sizeof(N) == 4;  // sums in the other solvers' order (rs_sums)
   constexpr int TH = kRsThreads, kWarps = TH / 32;
   constexpr int NW = sizeof(N) / 4;  // 32-bit words of a narrow value
   // a chunk's first word: index of its first cell, valid cells, chunk along z; its second
@@ -1342,7 +1524,7 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
   constexpr int kCnt = 18, kZc = 21;
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ double s_part[kRsMaxGroup][kQ];  // every CTA's sums
-  __shared__ Sum s_red[kWarps][kQ];
+  __shared__ double s_red[kOrder ? 1 : kWarps][kQ];
   __shared__ double s_tot[kQ], s_shift;
   __shared__ uint2 s_info[M * TH];
   __shared__ int s_cell[M * TH];  // first cell of a chunk in the mesh
@@ -1354,10 +1536,11 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
                            // z: the halo plane that takes it
     T *x, *b, *xp;
     const T* guess;
-    N* r;                  // the narrow true residual between its pass and the step loop
+    N* r;                  // the narrow true residual between its pass and the step loop (FP32
+                           // words in one CTA: in shared memory)
     unsigned long long* halo;  // grid: the group's tagged halo words, [CTA][parity][channel][hw]
-    unsigned long long* sums;  // grid: the group's tagged sums, [parity][CTA][kQ][2]
-    double inv;            // 1 / cells, or 1 / total weight on a graded mesh
+    unsigned long long* sums;  // grid: the group's tagged words of the sums (rs_sums; in
+                               // FP64 [parity][CTA][kQ][2])
   } s_g;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int G = a.rs_G, rank = (int)(blockIdx.x % (unsigned)G);
@@ -1386,6 +1569,7 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
     const int words = (zhi + (zcut ? bym * bxm : 0) + 3) & ~3;      // of a buffer
     const int bxy = bx * by, nzc = (bz + kRsZ - 1) / kRsZ, nch = bxy * nzc;
     const bool part = bz % kRsZ != 0;
+    [[maybe_unused]] const bool zz = md.cl_size > 0;    // order of a graded mesh's z terms
     // grid: room for the halo words of a CTA and channel
     const int hw = 2 * (nzcm * kRsZ * (bxm + bym) + (zcut ? bxm * bym : 0));
     const int nu = 2 * nzc * (bx + by), nw = zcut ? 2 * bxy : 0;  // halo units: chunks, words
@@ -1396,7 +1580,8 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
     // (local) or a tagged word of the neighbour's; and the word of this CTA's halo that
     // unit u of its own tagged words fills (kLocal: none)
     uint2* const s_push = (uint2*)(s_cz + (GR ? 2 * nzcm * kRsZ : 0));
-    uint32_t* const s_pull = (uint32_t*)(s_push + 2 * nzcm * (bxm + bym) + (zcut ? 2 * bxm * bym : 0));
+    const int nu_max = 2 * nzcm * (bxm + bym) + (zcut ? 2 * bxm * bym : 0);
+    uint32_t* const s_pull = (uint32_t*)(s_push + nu_max);
     constexpr uint32_t kLocal = 1u << 31;
 
     __syncthreads();  // the previous item's readers of s_g and s_info are done
@@ -1425,10 +1610,9 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
       s_g.b = (T*)md.b + f * C;
       s_g.xp = md.xp ? (T*)md.xp + f * C : nullptr;
       s_g.guess = md.guess ? (const T*)md.guess + f * C : nullptr;
-      s_g.r = (N*)md.q + f * C;
-      s_g.inv = GR ? 1.0 / md.z.wsum : 1.0 / (double)C;
-      s_g.sums = (unsigned long long*)md.d[0] + (size_t)grp * G * 2 * kQ * 2;
-      s_g.halo = (unsigned long long*)md.d[0] + (size_t)ngrp * G * 2 * kQ * 2 + (size_t)grp * G * 2 * P::n * hw * NW;
+      s_g.r = kOrder && G == 1 ? (N*)(s_pull + nu_max) : (N*)md.q + f * C;
+      s_g.sums = (unsigned long long*)md.d[0] + (size_t)grp * rs_sum_words(G);
+      s_g.halo = (unsigned long long*)md.d[0] + (size_t)ngrp * rs_sum_words(G) + (size_t)grp * G * 2 * P::n * hw * NW;
     }
     __syncthreads();
 #pragma unroll 1
@@ -1587,9 +1771,9 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
           }
         }
         if (!exchange(0, P::n)) return;
-        // ---- true residual (wide), its narrow copy to global memory, sums (each chunk's
-        //      in FP32, then compensated); the next chunk's b is loaded ahead
-        Sum sum[kQ] = {};
+        // ---- true residual (wide), its narrow copy to global memory, in FP64 the sums; the
+        //      next chunk's b is loaded ahead
+        [[maybe_unused]] N sum[kQ] = {};
         {
           const T cf[3] = {coef_w<T>(sp, 0), coef_w<T>(sp, 1), coef_w<T>(sp, 2)};
           T bn[kRsZ];
@@ -1617,32 +1801,28 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
             P::chunk(D0, D1, o + pr, bk);
             T below = P::one(D0, D1, (int)(in.y & 0xffffu));
             const T top = P::one(D0, D1, (int)(in.y >> 16));
-            N sr2 = N(0), sr = N(0), sb2 = N(0);
-            [[maybe_unused]] N sw = N(0);
 #pragma unroll
             for (int z = 0; z < kRsZ; ++z) {
               if (z < cnt) {
                 const T above = z + 1 < kRsZ && z + 1 < cnt ? c[z + 1 < kRsZ ? z + 1 : z] : top;
                 N rn;
                 if constexpr (GR)
-                  rn = Resid<T>::eval_z(cf, md.z.cz[ph] + 2 * (kz + z), c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
+                  rn = Resid<T>::eval_z(cf, md.z.cz[ph] + 2 * (kz + z), zz, c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
                 else
                   rn = Resid<T>::eval(cf, c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
                 out(z, rn);
-                sr2 += rn * rn;
-                sr += rn;
-                if constexpr (GR) sw += (N)md.z.w[kz + z] * rn;
-                if (round == 0) {
-                  const N b1 = W::narrow(bv[z]);
-                  sb2 += b1 * b1;
+                if constexpr (!kOrder) {
+                  sum[0] += rn * rn;
+                  sum[1] += rn;
+                  if constexpr (GR) sum[3] += (N)md.z.w[kz + z] * rn;
+                  if (round == 0) {
+                    const N b1 = W::narrow(bv[z]);
+                    sum[2] += b1 * b1;
+                  }
                 }
               }
               below = c[z];
             }
-            sum[0].add(sr2);
-            sum[1].add(sr);
-            if (round == 0) sum[2].add(sb2);
-            if constexpr (GR) sum[3].add(sw);
           };
           load_b(0);
           // rolled (x and q fill the registers): the residuals pass through global memory
@@ -1652,53 +1832,51 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
             chunk(m, [&](int z, N rn) { rg[z * nxy] = rn; });
           }
         }
-        // ---- the group's sums: warp (a reduce-scatter of the four), CTA, then the CTAs in
-        //      rank order
         ++rseq;
-        {
-          Sum s2[2];
-          const bool h4 = lane & 16, h3 = lane & 8;
+        if constexpr (kOrder) {
+          auto sums = [&](auto one) {
+            return rs_sums<T, GR, decltype(one)::value>(md, (const float*)s_g.r, s_g.b, round == 0, G, rank, (float*)s_part,
+                                                        s_g.sums, rseq, s_tot, &s_ok, a.ctl, a.spin_limit);
+          };
+          if (!(G == 1 ? sums(std::true_type{}) : sums(std::false_type{}))) return;
+        } else {
+          // ---- the group's sums: warp, CTA, then the CTAs in rank order
 #pragma unroll
-          for (int q = 0; q < 2; ++q) s2[q] = Sum::give(sum[q], sum[q + 2], h4, 16);
-          Sum t = Sum::give(s2[0], s2[1], h3, 8);
+          for (int q = 0; q < kQ; ++q) {
+            double t = sum[q];
 #pragma unroll
-          for (int o = 4; o > 0; o >>= 1) t.join(o);
-          if ((lane & 7) == 0) s_red[wid][(h4 ? 2 : 0) + (h3 ? 1 : 0)] = t;
-        }
-        __syncthreads();
-        if (wid == 0) {
-          // lane: sum lane >> 3 of warps lane & 7, ...
-          Sum t = s_red[lane & 7][lane >> 3];
-          for (int r = (lane & 7) + 8; r < kWarps; r += 8) t.plus(s_red[r][lane >> 3]);
-#pragma unroll
-          for (int o = 4; o > 0; o >>= 1) t.join(o);
-          if ((lane & 7) == 0) s_tot[lane >> 3] = t.d();
-          __syncwarp();
-          if (G > 1 && lane < kQ) {
-            const double v = s_tot[lane];
-            put2(s_g.sums + (((size_t)(rseq & 1) * G + rank) * kQ + lane) * 2, as_word(v, 0), as_word(v, 1), rseq);
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) s_red[wid][q] = t;
           }
-        }
-        if (G > 1) {
-          bool ok = true;
-          for (int t = tid; t < G * kQ; t += TH) {
-            const unsigned long long* p = s_g.sums + ((size_t)(rseq & 1) * G * kQ + t) * 2;
-            Tag2 v;
-            v.load(p);
-            Spin spin;
-            while (!v.is(rseq) && ok) {
-              ok = spin.go(a.ctl, a.spin_limit);
-              v.load(p);
-            }
-            of_words(s_part[t / kQ][t % kQ], (uint32_t)v.a, (uint32_t)v.b);
-          }
-          if (!ok) s_ok = 0;
           __syncthreads();
-          if (!s_ok) return;
+          if (tid < kQ) {
+            double t = 0.0;
+            for (int r = 0; r < kWarps; ++r) t += s_red[r][tid];
+            s_tot[tid] = t;
+            if (G > 1)
+              put2(s_g.sums + (((size_t)(rseq & 1) * G + rank) * kQ + tid) * 2, as_word(t, 0), as_word(t, 1), rseq);
+          }
+          if (G > 1) {
+            bool ok = true;
+            for (int t = tid; t < G * kQ; t += TH) {
+              const unsigned long long* p = s_g.sums + ((size_t)(rseq & 1) * G * kQ + t) * 2;
+              Tag2 v;
+              v.load(p);
+              Spin spin;
+              while (!v.is(rseq) && ok) {
+                ok = spin.go(a.ctl, a.spin_limit);
+                v.load(p);
+              }
+              of_words(s_part[t / kQ][t % kQ], (uint32_t)v.a, (uint32_t)v.b);
+            }
+            if (!ok) s_ok = 0;
+            __syncthreads();
+            if (!s_ok) return;
+          }
         }
         // the first warp of every CTA sums and decides: every CTA takes the same decision
         if (wid == 0) {
-          if (G > 1) {
+          if (!kOrder && G > 1) {
             const int q = lane >> 3;
             double t = 0.0;
             for (int r = lane & 7; r < G; r += 8) t += s_part[r][q];
@@ -1714,19 +1892,24 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
             double shift, rrp;
             if (GR) {
               // the shift keeps sum(w x) = sum(w b); |r - s|^2 = |r|^2 - 2 s sum r + C s^2
-              shift = zero ? 0.0 : s_tot[3] * s_g.inv;
+              shift = zero ? 0.0 : s_tot[3] / md.z.wsum;
               rrp = fmax(rr - 2.0 * shift * sr + (double)C * shift * shift, 0.0);
             } else {
-              shift = zero ? 0.0 : sr * s_g.inv;
-              rrp = fmax(rr - sr * (sr * s_g.inv), 0.0);
+              shift = zero ? 0.0 : sr / (double)C;
+              rrp = fmax(rr - sr * sr / (double)C, 0.0);
             }
             int k = 0;
             if (!zero && !(rrp <= a.rtol2 * bb)) {
               // |r_k| <= 2 sig^k |r_0|: enough steps for the tolerance, or for the reduction
-              // the narrow word can deliver in one round (the next round checks the true
-              // residual, so FP32 logarithms do)
-              const float need = fmaxf(0.5f * sqrtf((float)(a.rtol2 * bb / rrp)), (float)W::kFloor);
-              k = sp.sig > 0.0 ? (int)ceilf(logf(need) / logf((float)sp.sig)) : 1;
+              // the narrow word can deliver in one round (as the cluster solver forms the
+              // count where it would take the mesh, else as the streaming one)
+              if (md.cl_size > 0) {
+                const float need = fmaxf(0.5f * sqrtf((float)(a.rtol2 * bb / rrp)), (float)W::kFloor);
+                k = sp.sig > 0.0 ? (int)ceilf(logf(need) / logf((float)sp.sig)) : 1;
+              } else {
+                const double need = fmax(0.5 * sqrt(a.rtol2 * bb / rrp), W::kFloor);
+                k = sp.sig > 0.0 ? (int)ceil(log(need) / log(sp.sig)) : 1;
+              }
               if (k < 1) k = 1;
               if (k > kMaxStepsRound) k = kMaxStepsRound;
               if (total + k > a.max_iter) k = a.max_iter - total;
@@ -1821,7 +2004,7 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
               if constexpr (GR) {
                 const N* const cz = s_cz + 2 * ((int)(in.x >> kZc) * kRsZ + z);
                 const N tm = cz[0] * (below - cur), tp = cz[1] * (above - cur);
-                lap = (lap + tm) + tp;
+                lap = zz ? lap + (tm + tp) : (lap + tm) + tp;
               } else {
                 lap = lap + cfn[2] * ((below - cur) + (above - cur));
               }
@@ -1889,7 +2072,6 @@ int64_t smooth_units(int64_t C) { return (C + kThreads - 1) / kThreads; }
 // Room for the resident solver's tagged words behind the direction arrays: another such
 // array for meshes beyond a cluster, 4 MB for the small meshes of the FP64 form.
 static size_t rs_extra(int form, int64_t C) {
-  if (form == FORM_PLAIN) return 0;
   if (C > (int64_t)kClMaxCta * kClCells) return align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4));
   return form == FORM_FP64 ? (size_t)kSmoothTagBytes : 0;
 }
@@ -1909,7 +2091,7 @@ size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme) {
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf, void* work,
                   const DevState& st, int* iters_dev, double rtol, int max_iter, int n_tau,
                   int scheme, const double coef[3], const SmoothZ* z, cudaStream_t s,
-                  long long spin_limit, bool averaging) {
+                  long long spin_limit) {
   SmoothMesh m{};
   m.phi = phi;
   m.guess = guess;
@@ -1925,7 +2107,7 @@ int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, in
   if (z) m.z = *z;
   void* batch = (char*)work + align256(smooth_mesh_bytes(form, P.C, nf, scheme));
   return launch_smooth_batch(form, &m, 1, nf, batch, rtol, max_iter, n_tau, scheme, st.ctl,
-                             1 << 30, s, spin_limit, averaging);
+                             1 << 30, s, spin_limit);
 }
 
 size_t smooth_batch_bytes(int64_t B, int64_t U) {
@@ -2062,14 +2244,14 @@ struct RsPlan {
   size_t smem = 0, halo = 0;  // dynamic shared memory; halo words of a CTA and channel
 };
 
-// Bytes of a CTA's tagged words: two parities of the sums and of the halo words (the
-// double-float form has two channels of 4-byte words, FP64 one of 8 bytes).
-size_t rs_tag_bytes(size_t halo) { return 2 * kQ * 16 + halo * 4 * 8; }
+// Bytes of a group's tagged words: the sums, and for each CTA two parities of the halo words
+// (the double-float form has two channels of 4-byte words, FP64 one of 8 bytes).
+size_t rs_tag_bytes(int G, size_t halo) { return rs_sum_words(G) * 8 + (size_t)G * halo * 4 * 8; }
 
 // Fields of FP32 words that a thread's few chunks hold go to one CTA: no exchange at all,
 // and many meshes in one launch.
 bool rs_one_cta(int form, const SmoothMeshDev& m) {
-  return form == FORM_SPLIT &&
+  return form != FORM_FP64 &&
          (int64_t)m.nc[0] * m.nc[1] * ((m.nc[2] + kRsZ - 1) / kRsZ) <= kRsThreads * kRsChunks;
 }
 
@@ -2088,7 +2270,8 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
     const bool zcut = pz > 1 || m.per[2];
     const int64_t words = (nzc * (by + 2) * ((bx + 2) | 1) * kRsZ + (zcut ? 2 * bx * by : 0) + 3) / 4 * 4;
     const int64_t nu = 2 * nzc * (bx + by) + (zcut ? 2 * bx * by : 0);
-    const size_t smem = (2 * (size_t)words + 2 * (size_t)nzc * kRsZ) * word + (size_t)nu * 12;
+    const size_t smem = (2 * (size_t)words + 2 * (size_t)nzc * kRsZ) * word + (size_t)nu * 12 +
+                        (G == 1 && word == 4 ? m.C * 4 : 0);
     // a chunk's word holds 16 bits of index and 11 of its place along z
     if (smem > kRsSmem || words > 0xffff || nzc > 2000) return;
     const size_t halo = 2 * (size_t)(nzc * kRsZ * (bx + by) + (zcut ? bx * by : 0));
@@ -2102,7 +2285,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
     if (G > 1) {
       // every group's tagged sums and halo words live in the direction arrays of the
       // mesh's scratch
-      if ((int64_t)rs_tag_bytes(halo) * groups * G > m.halo_bytes) return;
+      if ((int64_t)rs_tag_bytes(G, halo) * groups > m.halo_bytes) return;
       t += 1.5 + 0.0018 * units + 0.00015 * planes;
     }
     const double cost = t * ((7 + groups - 1) / groups);  // waves of the averaging's seven fields
@@ -2150,7 +2333,7 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
   const int groups = pl.groups < a.nf ? pl.groups : a.nf;
   if ((int64_t)per_sm * nsm < (int64_t)groups * pl.G) return -3;
   // no tagged word of an earlier launch may pass for this one's: exchanges count from 1
-  const size_t bytes = rs_tag_bytes(pl.halo) * groups * pl.G;
+  const size_t bytes = rs_tag_bytes(pl.G, pl.halo) * groups;
   if (cudaMemsetAsync(m.d[0], 0, bytes, s) != cudaSuccess) return -3;
   SmoothBatchDev args = a;
   void* p[] = {&args};
@@ -2164,7 +2347,7 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
 
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit, bool averaging) {
+                        int max_blocks, cudaStream_t s, long long spin_limit) {
   if (B < 1 || B > kMaxBeds || nf < 1 || nf > kMaxF || (scheme != TAU_EULER && scheme != TAU_BDF2))
     return -1;
   // every mesh of a batch is graded or none is (one kernel instantiation per launch)
@@ -2175,14 +2358,12 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (nsm > max_blocks) nsm = max_blocks;
-  // FP32 words: meshes beyond one CTA that fit a cluster's shared memory take the cluster
-  // solver (one launch for every mesh of a cluster size).  Fields that fit one CTA and
-  // meshes that fit the whole chip take the resident solver, the rest the streaming grid
-  // solver.  The averaging of the FP32-force forms keeps the cluster and streaming solvers:
-  // the resident one differs from them in the last bits (~1e-11, far inside the tolerance),
-  // and an averaged solid fraction that rounds to another FP32 word changes the drag and
-  // with it a trajectory.  The plain form keeps them as the baseline.  The choice
-  // depends on the mesh alone, so a bed smooths the same way in any batch.
+  // FP32 words: fields that fit one CTA take the resident solver (10 x 10 x 20, seven fields:
+  // 440 us in a cluster solver's CTA, 250 here), larger meshes that fit a cluster's shared
+  // memory the cluster solver (one launch for every mesh of a cluster size), still larger
+  // ones the resident solver again where a cut of the whole chip fits, else the streaming grid
+  // solver.  In FP64 there is no cluster solver.  The choice depends on the mesh alone, and
+  // in FP32 words no bit of a result depends on it.
   struct Item {
     SmoothMeshDev m;
     RsPlan pl;
@@ -2192,13 +2373,9 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
   for (int b = 0; b < B; ++b) {
     Item it;
     smooth_mesh_layout(form, scheme, meshes[b], &it.m);
-    const bool rs = form == FORM_FP64 || (form == FORM_SPLIT && !averaging);
-    int cs = 0, planes = 0;
-    if (!rs || !rs_one_cta(form, it.m)) cluster_plan(form, it.m, &cs, &planes);
-    if (rs && cs == 0) it.pl = rs_plan(form, it.m, nsm);
-    if (cs > 0) {
-      it.m.cl_size = cs;
-      it.m.cl_planes = planes;
+    cluster_plan(form, it.m, &it.m.cl_size, &it.m.cl_planes);
+    if (it.m.cl_size == 0 || rs_one_cta(form, it.m)) it.pl = rs_plan(form, it.m, nsm);
+    if (it.m.cl_size > 0 && it.pl.G != 1) {
       mc.push_back(it.m);
     } else if (it.pl.G > 0) {
       it.m.rs_G = it.pl.G;
@@ -2272,11 +2449,16 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
       c.rs_G = pl.G;
       if (form == FORM_SPLIT)
         rc = gr ? launch_rs<dd, true>(c, pl, mr[i0].m, nsm, s) : launch_rs<dd, false>(c, pl, mr[i0].m, nsm, s);
+      else if (form == FORM_PLAIN)
+        rc = gr ? launch_rs<float, true>(c, pl, mr[i0].m, nsm, s) : launch_rs<float, false>(c, pl, mr[i0].m, nsm, s);
       else
         rc = gr ? launch_rs<double, true>(c, pl, mr[i0].m, nsm, s) : launch_rs<double, false>(c, pl, mr[i0].m, nsm, s);
       if (rc) {
         cudaGetLastError();
-        for (size_t i = i0; i < i1; ++i) mg.push_back(mr[i].m);
+        for (size_t i = i0; i < i1; ++i) {
+          mg.push_back(mr[i].m);
+          mg.back().cl_size = mg.back().cl_planes = 0;
+        }
         rc = 0;
       }
       i0 = i1;

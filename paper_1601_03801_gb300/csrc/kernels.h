@@ -191,7 +191,7 @@ struct alignas(16) SmoothMeshDev {
   int64_t C, u0, nu;  // cells, first unit, units
   int32_t nc[3], per[3];
   uint64_t div_x, div_xy;            // ceil(2^64 / nx), ceil(2^64 / (nx ny)) (0: divisor 1)
-  int32_t cl_size, cl_planes;        // cluster solver: CTAs, z-planes per CTA (0: not this solver)
+  int32_t cl_size, cl_planes;        // cluster solver's CTAs, z-planes per CTA (0: does not fit)
   int64_t halo_bytes;                // resident solver: room for halo words from d[0] on
   int32_t rs_G, rs_px, rs_py, rs_pz;  // resident solver: CTAs, cuts per axis (0: streaming solver)
   SmoothSpec sp[2];  // [0]: backward-Euler steps (coef); [1]: BDF2 steps (2/3 coef)
@@ -232,17 +232,16 @@ size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme);
 size_t smooth_batch_bytes(int64_t B, int64_t U);
 // Smooth every mesh's nf fields in place by n_tau pseudo-steps of the scheme;
 // batch_work: smooth_batch_bytes(B, sum of units) bytes.  Returns 0, -1 (bad sizes)
-// or -3 (launch failed).  averaging: the result feeds the drag law.
+// or -3 (launch failed).
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins,
-                        bool averaging = false);
+                        int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins);
 // Single mesh: work holds smooth_work_bytes(form, C, nf, scheme) = mesh + batch scratch.
 size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme);
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf,
                   void* work, const DevState& st, int* iters_dev, double rtol, int max_iter,
                   int n_tau, int scheme, const double coef[3], const SmoothZ* z,
-                  cudaStream_t s, long long spin_limit = kBarrierSpins, bool averaging = false);
+                  cudaStream_t s, long long spin_limit = kBarrierSpins);
 void launch_average_out(int form, const void* phi, const DevParams& P, void* ufe, double* eps,
                         double* Us, double* F, cudaStream_t s);
 void launch_phi_convert(int form, const void* phi, double* out, int64_t n, int to_double,
