@@ -888,6 +888,17 @@ __global__ void k_export(DevState st, int what, double* out) {
   }
 }
 
+// fdbg [4][N][3] in sorted order -> caller order: words read in a row, written three by three
+__global__ void k_forces_out(DevState st, double* out) {
+  const int pb = st.ctl->pb;
+  const int64_t n3 = 3 * st.N;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n3; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / 3, to = 3 * (int64_t)st.uid[pb][i] + (e - 3 * i);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k * n3 + to] = st.fdbg[k * n3 + e];
+  }
+}
+
 __global__ void k_nbr_counts(DevState st, int64_t* counts) {
   const int pb = st.ctl->pb, nl = st.ctl->nl;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < st.N;
@@ -1070,6 +1081,10 @@ void launch_export(int form, const DevState& st, int what, double* out, cudaStre
     case FORM_PLAIN: k_export<FORM_PLAIN><<<g, 256, 0, s>>>(st, what, out); break;
     default: k_export<FORM_FP64><<<g, 256, 0, s>>>(st, what, out); break;
   }
+}
+
+void launch_forces_out(const DevState& st, double* out, cudaStream_t s) {
+  k_forces_out<<<grid_for(3 * st.N, 256), 256, 0, s>>>(st, out);
 }
 
 void launch_neighbors_export(const DevState& st, int64_t* counts, cudaStream_t s) {

@@ -99,6 +99,7 @@ void launch_export(int form, const DevState& st, int what, double* out, cudaStre
 void launch_import(int form, const DevState& st, const double* x, const double* v,
                    const double* w, const double* d, const double* rho, const DevParams& P,
                    cudaStream_t s);
+void launch_forces_out(const DevState& st, double* out, cudaStream_t s);
 void launch_neighbors_export(const DevState& st, int64_t* counts, cudaStream_t s);
 void launch_neighbors_fill(const DevState& st, const int64_t* offsets, int64_t* out,
                            cudaStream_t s);
