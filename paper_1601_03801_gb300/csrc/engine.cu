@@ -99,6 +99,8 @@ struct sedi_handle {
   bool ens_dirty = true;          // a bed's buffers changed: rebuild the table
   int ens_variant = SUBSTEP_B128_LOOP;  // launch shape of the batched substep
   int* ens_done = nullptr;        // substeps completed by the last persistent launch
+  SmoothSide ens_side{};          // streams of the batched smoother's launches
+  bool ens_side_set = false;
   bool ens_fresh = false;         // the batched averaging is newer than the last step
 };
 
@@ -1159,6 +1161,11 @@ void sedi_destroy(sedi_handle* h) {
   if (h->part_block.p) cudaFree(h->part_block.p);
   if (h->bin_block.p) cudaFree(h->bin_block.p);
   if (h->ctl_host) cudaFreeHost(h->ctl_host);
+  if (h->ens_side.fork) cudaEventDestroy(h->ens_side.fork);
+  for (int k = 0; k < kSmoothSides; ++k) {
+    if (h->ens_side.s[k]) cudaStreamDestroy(h->ens_side.s[k]);
+    if (h->ens_side.join[k]) cudaEventDestroy(h->ens_side.join[k]);
+  }
   free_list(h->mesh_allocs);
   if (h->dstage) cudaFree(h->dstage);
   for (void* p : {(void*)h->cnn_master, (void*)h->cnn_m, (void*)h->cnn_v, (void*)h->cnn_grad,
@@ -1858,6 +1865,18 @@ static int ens_step(sedi_handle* h, int n) {
 
 // Deposition and smoothing of every bed in batched launches; the smoothed eps
 // feeds each bed's drag.  Outputs stay on the device.
+static int ens_streams(sedi_handle* h) {
+  if (h->ens_side_set) return 0;
+  SmoothSide& e = h->ens_side;
+  if (!e.fork) CK(cudaEventCreateWithFlags(&e.fork, cudaEventDisableTiming));
+  for (int k = 0; k < kSmoothSides; ++k) {
+    if (!e.s[k]) CK(cudaStreamCreateWithFlags(&e.s[k], cudaStreamNonBlocking));
+    if (!e.join[k]) CK(cudaEventCreateWithFlags(&e.join[k], cudaEventDisableTiming));
+  }
+  h->ens_side_set = true;
+  return 0;
+}
+
 static int ens_average(sedi_handle* h) {
   int rc = ens_finalize(h);
   if (rc) return rc;
@@ -1868,6 +1887,7 @@ static int ens_average(sedi_handle* h) {
       for (int k = 0; k < 5; ++k) h->avg_ev.push_back(new_event());
     CK(cudaEventRecord(h->avg_ev[0], h->stream));
   }
+  if ((rc = ens_streams(h))) return rc;
   launch_deposit_ens(h->form, h->ens, h->stream);
   if (h->prm.profile) CK(cudaEventRecord(h->avg_ev[1], h->stream));
   std::vector<SmoothMesh> m(B);
@@ -1891,7 +1911,7 @@ static int ens_average(sedi_handle* h) {
   const double rtol = h->form == FORM_PLAIN ? std::max(h->prm.cg_rtol, 2e-6) : h->prm.cg_rtol;
   if (launch_smooth_batch(h->form, m.data(), B, 7, h->ens_smooth, rtol, h->prm.cg_max_iter,
                           h->prm.n_tau, h->prm.tau_scheme, h->st.ctl, 1 << 30, h->stream,
-                          h->barrier_spins))
+                          h->barrier_spins, &h->ens_side))
     return fail(h, SEDI_ECUDA, "cooperative launch of the batched smoother failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
   launch_eps_out_ens(h->form, h->ens, h->stream);

@@ -2207,9 +2207,9 @@ int launch_cluster(const SmoothBatchDev& a, int csize, cudaStream_t s) {
   cfg.gridDim = dim3(csize * 64);
   int ncl = 0;
   if (cudaOccupancyMaxActiveClusters(&ncl, (void*)k_smooth_cl<T, GR>, &cfg) != cudaSuccess || ncl < 1) return -3;
-  const int64_t items = (int64_t)a.B * a.nf;
-  if (ncl > items) ncl = (int)items;
-  cfg.gridDim = dim3(csize * ncl);
+  // a cluster an item: clusters beyond the resident ones start as others end, so long and
+  // short fields, and launches of other cluster sizes beside this one, share the SMs
+  cfg.gridDim = dim3((unsigned)(csize * a.B * a.nf));
   return cudaLaunchKernelEx(&cfg, k_smooth_cl<T, GR>, a) == cudaSuccess ? 0 : -3;
 }
 
@@ -2347,7 +2347,7 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
 
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit) {
+                        int max_blocks, cudaStream_t s, long long spin_limit, const SmoothSide* side) {
   if (B < 1 || B > kMaxBeds || nf < 1 || nf > kMaxF || (scheme != TAU_EULER && scheme != TAU_BDF2))
     return -1;
   // every mesh of a batch is graded or none is (one kernel instantiation per launch)
@@ -2387,10 +2387,11 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
       mg.push_back(it.m);
     }
   }
-  // cluster meshes grouped by cluster size (one launch per size), resident ones with the
+  // cluster meshes grouped by cluster size (one launch per size, the largest first: the
+  // small clusters fit between them), resident ones with the
   // meshes of one CTA first (one launch for all)
   std::stable_sort(mc.begin(), mc.end(),
-                   [](const SmoothMeshDev& x, const SmoothMeshDev& y) { return x.cl_size < y.cl_size; });
+                   [](const SmoothMeshDev& x, const SmoothMeshDev& y) { return x.cl_size > y.cl_size; });
   std::stable_sort(mr.begin(), mr.end(), [](const Item& x, const Item& y) { return (x.pl.G == 1) > (y.pl.G == 1); });
   char* p = (char*)batch_work;
   SmoothBatchDev a{};
@@ -2411,18 +2412,33 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
     for (const auto& it : mr) tab.push_back(it.m);
     if (cudaMemcpyAsync(tab_c, tab.data(), tab.size() * sizeof(SmoothMeshDev), cudaMemcpyHostToDevice, s) != cudaSuccess)
       return -3;
+    // The launches of the cluster sizes run side by side where there are streams for it: a
+    // GPC's SMs hold one cluster of 11 CTAs and one of 8 at once, and no launch waits
+    // for the last cluster of another (48 beds of 16^3 to 48^3 cells, seven fields: 9.8 ms
+    // one after the other, 8.6 side by side).
+    const bool fork = side && !mc.empty() && mc.front().cl_size != mc.back().cl_size;
+    if (fork && cudaEventRecord(side->fork, s) != cudaSuccess) return -3;
+    unsigned used = 0;  // side streams with work
+    int lane = 0;
     for (size_t i0 = 0; i0 < mc.size();) {
       size_t i1 = i0;
       while (i1 < mc.size() && mc[i1].cl_size == mc[i0].cl_size) ++i1;
+      cudaStream_t on = s;
+      if (fork) {
+        on = side->s[lane];
+        if (!(used >> lane & 1u) && cudaStreamWaitEvent(on, side->fork, 0) != cudaSuccess) return -3;
+        used |= 1u << lane;
+        lane = (lane + 1) % kSmoothSides;
+      }
       SmoothBatchDev c = a;
       c.mesh = tab_c + i0;
       c.B = (int32_t)(i1 - i0);
       if (gr)
-        rc = form == FORM_SPLIT ? launch_cluster<dd, true>(c, mc[i0].cl_size, s)
-                                : launch_cluster<float, true>(c, mc[i0].cl_size, s);
+        rc = form == FORM_SPLIT ? launch_cluster<dd, true>(c, mc[i0].cl_size, on)
+                                : launch_cluster<float, true>(c, mc[i0].cl_size, on);
       else
-        rc = form == FORM_SPLIT ? launch_cluster<dd, false>(c, mc[i0].cl_size, s)
-                                : launch_cluster<float, false>(c, mc[i0].cl_size, s);
+        rc = form == FORM_SPLIT ? launch_cluster<dd, false>(c, mc[i0].cl_size, on)
+                                : launch_cluster<float, false>(c, mc[i0].cl_size, on);
       if (rc) {
         // a device without this cluster shape: these meshes take the streaming solver
         cudaGetLastError();
@@ -2435,6 +2451,10 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
       }
       i0 = i1;
     }
+    for (int k = 0; k < kSmoothSides; ++k)
+      if (used >> k & 1u)
+        if (cudaEventRecord(side->join[k], side->s[k]) != cudaSuccess || cudaStreamWaitEvent(s, side->join[k], 0) != cudaSuccess)
+          return -3;
     for (size_t i0 = 0; i0 < mr.size();) {
       // every mesh of one CTA in one launch, the larger ones one by one
       size_t i1 = i0 + 1;

@@ -227,6 +227,13 @@ constexpr int kSmoothSums = 4;
 // the resident solver's tagged words of a small FP64 mesh (see smooth_mesh_bytes)
 constexpr int kSmoothTagBytes = 4 << 20;
 
+// Streams beside the caller's for the launches of a batch, and their events.
+constexpr int kSmoothSides = 6;
+struct SmoothSide {
+  cudaStream_t s[kSmoothSides];
+  cudaEvent_t fork, join[kSmoothSides];
+};
+
 int64_t smooth_units(int64_t C);
 // scratch of one mesh, and of the batch tables
 size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme);
@@ -236,7 +243,8 @@ size_t smooth_batch_bytes(int64_t B, int64_t U);
 // or -3 (launch failed).
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins);
+                        int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins,
+                        const SmoothSide* side = nullptr);
 // Single mesh: work holds smooth_work_bytes(form, C, nf, scheme) = mesh + batch scratch.
 size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme);
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf,
