@@ -127,14 +127,18 @@ __device__ __forceinline__ uint32_t pair_of(__nv_bfloat16 a, __nv_bfloat16 b) {
 }
 
 struct Tiling {
-  int nx, ny;     // tiles along x and y
-  int64_t n;      // tiles
+  unsigned nx, ny;  // tiles along x and y
+  unsigned n;       // tiles (a mesh has fewer than 2^31 cells)
+  __device__ __forceinline__ int3 at(unsigned tile, int ty, int tz) const {
+    const unsigned q = tile / nx, z = q / ny;
+    return make_int3((int)(tile - q * nx) * kTX, (int)(q - z * ny) * ty, (int)z * tz);
+  }
 };
 Tiling tiling(const Grid3& g, int ty, int tz) {
   Tiling t;
   t.nx = (g.nx + kTX - 1) / kTX;
   t.ny = (g.ny + ty - 1) / ty;
-  t.n = (int64_t)t.nx * t.ny * ((g.nz + tz - 1) / tz);
+  t.n = t.nx * t.ny * ((g.nz + tz - 1) / tz);
   return t;
 }
 
@@ -194,9 +198,9 @@ __global__ void __launch_bounds__(kConvThreads)
   for (int n = 0; n < NT; ++n)
 #pragma unroll
     for (int e = 0; e < 2; ++e) bv[n][e] = bias ? bias[n * 8 + 2 * tig + e] : 0.0f;
-  for (int64_t tile = blockIdx.x; tile < tl.n; tile += gridDim.x) {
-    const int x0 = (int)(tile % tl.nx) * kTX, y0 = (int)((tile / tl.nx) % tl.ny) * TY,
-              z0 = (int)(tile / ((int64_t)tl.nx * tl.ny)) * TZ;
+  for (unsigned tile = blockIdx.x; tile < tl.n; tile += gridDim.x) {
+    const int3 t0 = tl.at(tile, TY, TZ);
+    const int x0 = t0.x, y0 = t0.y, z0 = t0.z;
     stage_halo<KC, NP, TY, TZ, kConvThreads>(sx, in, g, x0, y0, z0);
     cp_commit();
     cp_wait<0>();
@@ -300,9 +304,9 @@ __global__ void __launch_bounds__(kConv1Threads)
   __shared__ float4 sx[HV];
   for (int k = threadIdx.x; k < 27 * 4 * 8; k += kConv1Threads) sw[k] = ((const float4*)wt)[k];
   const int n8 = threadIdx.x & 3, y = (threadIdx.x >> 2) & 7, z = threadIdx.x >> 5;
-  for (int64_t tile = blockIdx.x; tile < tl.n; tile += gridDim.x) {
-    const int x0 = (int)(tile % tl.nx) * kTX, y0 = (int)((tile / tl.nx) % tl.ny) * TY,
-              z0 = (int)(tile / ((int64_t)tl.nx * tl.ny)) * TZ;
+  for (unsigned tile = blockIdx.x; tile < tl.n; tile += gridDim.x) {
+    const int3 t0 = tl.at(tile, TY, TZ);
+    const int x0 = t0.x, y0 = t0.y, z0 = t0.z;
     for (int k = threadIdx.x; k < HV; k += kConv1Threads) {
       const int64_t q = nb_of(g, x0 + k % kHX - 1, y0 + (k / kHX) % HY - 1, z0 + k / (kHX * HY) - 1);
       const uint2 u = q < 0 ? make_uint2(0u, 0u) : *(const uint2*)(x + q * 16);
@@ -397,10 +401,10 @@ __global__ void __launch_bounds__(Wg<MT, NT>::threads)
 #pragma unroll
   for (int k = 0; k < 3 * NT * 4; ++k) sums[k * W::threads] = 0.0f;
 
-  auto stage = [&](int64_t tile, int buf) {
+  auto stage = [&](unsigned tile, int buf) {
     const uint32_t sa = sb + buf * (W::bytes_a + W::bytes_b);
-    const int x0 = (int)(tile % tl.nx) * kTX, y0 = (int)((tile / tl.nx) % tl.ny) * TY,
-              z0 = (int)(tile / ((int64_t)tl.nx * tl.ny)) * TZ;
+    const int3 t0 = tl.at(tile, TY, TZ);
+    const int x0 = t0.x, y0 = t0.y, z0 = t0.z;
     constexpr int CH = KA / 8, ROW = CH * NP;
     for (int k = threadIdx.x; k < W::TV * ROW; k += W::threads) {
       const int v = k / ROW, c = k % ROW;
@@ -413,9 +417,9 @@ __global__ void __launch_bounds__(Wg<MT, NT>::threads)
   };
 
   int buf = 0;
-  if ((int64_t)blockIdx.x < tl.n) stage(blockIdx.x, 0);
+  if (blockIdx.x < tl.n) stage(blockIdx.x, 0);
   cp_commit();
-  for (int64_t tile = blockIdx.x; tile < tl.n; tile += gridDim.x, buf ^= 1) {
+  for (unsigned tile = blockIdx.x; tile < tl.n; tile += gridDim.x, buf ^= 1) {
     if (tile + gridDim.x < tl.n) stage(tile + gridDim.x, buf ^ 1);
     cp_commit();
     cp_wait<1>();
