@@ -296,15 +296,14 @@ def tuned_launch(st):
             "chosen_by": "autotuner"}
 
 
-def launches_per_step(variant, rebuilds, steps, cells):
+def launches_per_step(variant, rebuilds, steps):
     """Kernels of one step: the graph's rebuild check, 20 substeps of one kernel (two
     with the pair list), 16 per list rebuild taken (the split form keeps the pair
     list -- counts, scan, fill -- whatever the variant), then deposition,
-    fixed point -> smoothing word, the smoother (the cluster solver: one launch; the
-    grid solver: barrier reset + cooperative launch) and the outputs."""
+    fixed point -> smoothing word, the smoother (one launch, of the cluster or the on-chip
+    solver) and the outputs."""
     per_sub = 2 if variant in PAIR_VARIANTS else 1
-    per_avg = 4 if cells <= 131072 else 5
-    return steps * (1 + per_sub * SUBSTEPS + per_avg) + 16 * rebuilds
+    return steps * (1 + per_sub * SUBSTEPS + 4) + 16 * rebuilds
 
 
 def gpu_arm(args):
@@ -376,7 +375,7 @@ def gpu_arm(args):
                            "parallelism": "independent bed per GPU" if world > 1 else "1 GPU"},
                 "phases_ms_per_step": phases, "rebuilds_in_timed_region": int(rebuilds),
                 "roofline": roof, "e2e": e2e,
-                "gpu_launches": int(launches_per_step(variant, rebuilds, args.steps, C)),
+                "gpu_launches": int(launches_per_step(variant, rebuilds, args.steps)),
                 "clocks": m["clocks"], "cpu_baseline": cpu, "other_forms": plain, **extra}
         print(json.dumps(line))
     if world > 1:

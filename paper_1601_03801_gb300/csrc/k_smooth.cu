@@ -2069,10 +2069,12 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 int64_t smooth_units(int64_t C) { return (C + kThreads - 1) / kThreads; }
 
-// Room for the resident solver's tagged words behind the direction arrays: another such
-// array for meshes beyond a cluster, 4 MB for the small meshes of the FP64 form.
+// Room for the resident solver's tagged words behind the direction arrays: what these lack
+// of 24 MB for meshes beyond a cluster (150 CTAs of 160 KB), 4 MB for the small meshes of
+// the FP64 form.
 static size_t rs_extra(int form, int64_t C) {
-  if (C > (int64_t)kClMaxCta * kClCells) return align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4));
+  const size_t have = 2 * align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4)), want = 24 << 20;
+  if (C > (int64_t)kClMaxCta * kClCells) return have < want ? want - have : 0;
   return form == FORM_FP64 ? (size_t)kSmoothTagBytes : 0;
 }
 
