@@ -25,6 +25,7 @@ using namespace sedi;
 struct Block {
   char* p = nullptr;
   size_t n = 0;
+  int64_t epoch = 0;  // the handle's stream_epoch when it was filled
 };
 
 struct sedi_handle {
@@ -44,6 +45,7 @@ struct sedi_handle {
   DevState st{};
   DevParams P{};
   DevMesh mesh{};
+  int64_t stream_epoch = 0;        // changes of the stream so far
   Block part_block;                // per-particle buffers
   Block bin_block;                 // link-cell bins (resized when the bin size changes)
   std::vector<void*> mesh_allocs;
@@ -139,13 +141,15 @@ using Parts = std::vector<std::pair<void**, size_t>>;  // buffers and their byte
 
 // Place the buffers in the block, each on a 256-byte boundary.  The block is kept while they
 // fill most of it (loading 200,000 spheres into a handle that has as many spent 3.0 of its
-// 4.9 ms in 43 frees and allocations), else allocated anew.  Either way no earlier work of
-// any stream is left on it: the wait is the one that freeing it has.
+// 4.9 ms in 43 frees and allocations), else allocated anew.  Either way no earlier work is
+// left on it: a block is used by work of the handle's stream alone, so the wait is for that
+// stream, or, where the stream has changed since, the one that freeing the block has.  (A
+// wait for the whole device is refused while any thread captures a graph.)
 int fill_block(sedi_handle* h, Block& b, const Parts& parts) {
   auto room = [](size_t bytes) { return (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255; };
   size_t n = 0;
   for (const auto& p : parts) n += room(p.second);
-  if (b.n < n || b.n > n + n / 4 + (1 << 20)) {
+  if (b.n < n || b.n > n + n / 4 + (1 << 20) || b.epoch != h->stream_epoch) {
     if (b.p) cudaFree(b.p);
     b = Block{};
     const cudaError_t e = cudaMalloc((void**)&b.p, n);
@@ -154,8 +158,9 @@ int fill_block(sedi_handle* h, Block& b, const Parts& parts) {
       return fail(h, SEDI_ENOMEM, "cudaMalloc(%zu) failed: %s", n, cudaGetErrorString(e));
     }
     b.n = n;
+    b.epoch = h->stream_epoch;
   } else {
-    CK(cudaDeviceSynchronize());
+    CK(cudaStreamSynchronize(h->stream));
   }
   char* at = b.p;
   for (const auto& p : parts) {
@@ -1179,7 +1184,10 @@ void sedi_destroy(sedi_handle* h) {
 
 int sedi_set_stream(sedi_handle* h, void* s) {
   if (!h) return SEDI_EINVAL;
-  if ((cudaStream_t)s != h->stream) clear_graphs(h);
+  if ((cudaStream_t)s != h->stream) {
+    clear_graphs(h);
+    ++h->stream_epoch;
+  }
   h->stream = (cudaStream_t)s;
   for (sedi_handle* b : h->beds) sedi_set_stream(b, s);
   return 0;
