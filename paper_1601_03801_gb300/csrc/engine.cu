@@ -2363,14 +2363,24 @@ struct CkHeader {
 int ck_write(FILE* f, const void* p, size_t n) { return fwrite(p, 1, n, f) == n ? 0 : -1; }
 int ck_read(FILE* f, void* p, size_t n) { return fread(p, 1, n, f) == n ? 0 : -1; }
 
+// A copy on the handle's stream, waited for: behind what is queued there (the zeros of newly
+// placed buffers, steps still running) and ahead of what follows, which a copy on the
+// default stream is not.
+int copy_wait(sedi_handle* h, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {
+  CK(cudaMemcpyAsync(dst, src, bytes, kind, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return 0;
+}
+
 int dev_io(sedi_handle* h, FILE* f, void* dptr, size_t bytes, bool save) {
   std::vector<char> buf(bytes);
+  int rc;
   if (save) {
-    CK(cudaMemcpy(buf.data(), dptr, bytes, cudaMemcpyDeviceToHost));
+    if ((rc = copy_wait(h, buf.data(), dptr, bytes, cudaMemcpyDeviceToHost))) return rc;
     if (ck_write(f, buf.data(), bytes)) return fail(h, SEDI_EIO, "checkpoint write failed");
   } else {
     if (ck_read(f, buf.data(), bytes)) return fail(h, SEDI_EIO, "checkpoint read failed");
-    CK(cudaMemcpy(dptr, buf.data(), bytes, cudaMemcpyHostToDevice));
+    if ((rc = copy_wait(h, dptr, buf.data(), bytes, cudaMemcpyHostToDevice))) return rc;
   }
   return 0;
 }
@@ -2379,8 +2389,8 @@ int state_io(sedi_handle* h, FILE* f, bool save) {
   const int64_t N = h->N, C = h->P.C, cap = h->P.cap;
   const size_t q = quad_bytes(h->form), fq = fquad_bytes(h->form), w = word_bytes(h->form);
   Ctl c;
-  CK(cudaMemcpy(&c, h->st.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost));
   int rc;
+  if ((rc = copy_wait(h, &c, h->st.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost))) return rc;
   DevState& s = h->st;
   struct Item { void* p; size_t n; };
   std::vector<Item> items = {
@@ -2402,7 +2412,7 @@ int state_io(sedi_handle* h, FILE* f, bool save) {
     in.st = c.st;
     in.pb = c.pb;
     in.nl = c.nl;
-    CK(cudaMemcpy(h->st.ctl, &in, sizeof(Ctl), cudaMemcpyHostToDevice));
+    if ((rc = copy_wait(h, h->st.ctl, &in, sizeof(Ctl), cudaMemcpyHostToDevice))) return rc;
   }
   return 0;
 }
@@ -2465,9 +2475,10 @@ static int load_from(sedi_handle* h, FILE* f) {
   if (!rc) {
     h->gp_default = gpd != 0;
     // the fluid fields back on the device (the mesh words come with the state below)
-    CK(cudaMemcpy(h->fdev, h->U.data(), 24 * C, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->fdev + 3 * C, h->gp.data(), 24 * C, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->fdev + 6 * C, h->du.data(), 24 * C, cudaMemcpyHostToDevice));
+    if ((rc = copy_wait(h, h->fdev, h->U.data(), 24 * C, cudaMemcpyHostToDevice)) ||
+        (rc = copy_wait(h, h->fdev + 3 * C, h->gp.data(), 24 * C, cudaMemcpyHostToDevice)) ||
+        (rc = copy_wait(h, h->fdev + 6 * C, h->du.data(), 24 * C, cudaMemcpyHostToDevice)))
+      return rc;
     h->fluid_host_stale = false;
     double rmax = 0;
     for (double di : d) rmax = std::max(rmax, 0.5 * di);
@@ -2487,8 +2498,8 @@ static int load_from(sedi_handle* h, FILE* f) {
     h->rho_host = rho;
     h->ids = ids;
     Ctl zero{};
-    cudaMemcpy(h->st.ctl, &zero, sizeof(Ctl), cudaMemcpyHostToDevice);
-    rc = state_io(h, f, false);
+    rc = copy_wait(h, h->st.ctl, &zero, sizeof(Ctl), cudaMemcpyHostToDevice);
+    if (!rc) rc = state_io(h, f, false);
   }
   if (rc) return rc;
   // the pair list follows the loaded neighbour lists
