@@ -3,11 +3,9 @@
 // device), orchestration of the averaging, import/export in caller order and
 // checkpoints.  All arithmetic of the method runs in the kernels of k_*.cu.
 #include <cuda_runtime.h>
-#include <sys/mman.h>
 #include <unistd.h>
 
 #include <algorithm>
-#include <cerrno>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -21,10 +19,6 @@
 #include "../../include/sedi.h"
 #include "common.cuh"
 #include "kernels.h"
-
-#ifndef MADV_POPULATE_WRITE
-#define MADV_POPULATE_WRITE 23  // Linux 5.14
-#endif
 
 using namespace sedi;
 
@@ -360,20 +354,30 @@ int copy_in(sedi_handle* h, void* dst, const void* src, size_t bytes, int mem) {
   return 0;
 }
 
-// Map the pages of a large host output: a copy into pages that the process has not touched
-// yet maps them one by one from the GPU's side (four arrays of 24 MB 60 ms, 2.5 with the
-// pages in place).  Content stays; where it cannot be done the copy is merely slower.
+// Whether a host output is large and the process's own pageable memory (see map_pages).
+bool pageable(const void* dst, size_t bytes) {
+  if (bytes < (256u << 10)) return false;  // the heap's pages are in place mostly
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeUnregistered;
+}
+
+// Map the pages of a pageable output that is about to be overwritten: a copy into pages that
+// the process has not touched yet maps them one by one from the GPU's side (four arrays of
+// 24 MB 60 ms, 2.5 with the pages in place).  By a store to each: a load would map the zero
+// page first, and a system call costs 4 us where the pages are in place, these stores nothing.
 void map_pages(void* dst, size_t bytes) {
-  if (bytes < (256u << 10)) return;  // the heap's pages are in place mostly
-  static const uintptr_t page = (uintptr_t)std::max(4096l, sysconf(_SC_PAGESIZE));
-  const uintptr_t lo = (uintptr_t)dst & ~(page - 1), hi = ((uintptr_t)dst + bytes + page - 1) & ~(page - 1);
-  const int saved = errno;
-  madvise((void*)lo, hi - lo, MADV_POPULATE_WRITE);
-  errno = saved;
+  static const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+  volatile char* const p = (volatile char*)dst;
+  for (size_t k = 0; k < bytes; k += page) p[k] = 0;
+  p[bytes - 1] = 0;
 }
 
 int copy_out(sedi_handle* h, void* dst, const void* src, size_t bytes, int mem) {
-  if (mem != SEDI_MEM_DEVICE) map_pages(dst, bytes);
+  if (mem != SEDI_MEM_DEVICE && pageable(dst, bytes)) map_pages(dst, bytes);
   CK(cudaMemcpyAsync(dst, src, bytes, mem == SEDI_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
   return 0;
 }
@@ -2286,9 +2290,15 @@ int sedi_compute_forces(sedi_handle* h, int32_t bed, double* fc, double* fl, dou
       if (outs[k]) std::memcpy(outs[k], tmp.data() + 3 * N * k, 24 * N);
     return 0;
   }
+  bool map[4];  // asked while the kernels run
+  for (int k = 0; k < 4; ++k) map[k] = mem != SEDI_MEM_DEVICE && outs[k] && pageable(outs[k], 24 * N);
   if ((rc = sync_status(h))) return rc;
-  for (int k = 0; k < 4; ++k)
-    if (outs[k] && (rc = copy_out(h, outs[k], h->dstage + 3 * N * k, 24 * N, mem))) return rc;
+  const cudaMemcpyKind kind = mem == SEDI_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  for (int k = 0; k < 4; ++k) {
+    if (!outs[k]) continue;
+    if (map[k]) map_pages(outs[k], 24 * N);
+    CK(cudaMemcpyAsync(outs[k], h->dstage + 3 * N * k, 24 * N, kind, h->stream));
+  }
   CK(cudaStreamSynchronize(h->stream));
   return 0;
 }
