@@ -1115,10 +1115,10 @@ int sedi_create(const sedi_params* p, sedi_handle** out) {
   }
   h->form = p->precision_form;
   h->variant = p->substep_variant >= 0 && h->form != FORM_FP64 ? p->substep_variant : SUBSTEP_B128_LOOP;
-  // a lower limit on the smoother's grid-barrier waits, for failure-detection tests
+  // a lower limit on the smoother's waits between blocks, for failure-detection tests
   if (const char* lim = std::getenv("SEDI_BARRIER_SPIN_LIMIT")) {
     const long long v = std::atoll(lim);
-    if (v > 0) h->barrier_spins = v;
+    if (v > 0) h->barrier_spins = std::min(v, kBarrierSpins);
   }
   fill_params(h);
   const int64_t C = h->P.C;

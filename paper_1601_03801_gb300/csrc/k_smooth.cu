@@ -32,7 +32,7 @@
 // is a per-unit partial sum followed by a per-mesh sum over its units in unit
 // order, so a mesh's result does not depend on the grid size or on the other
 // meshes of the batch: a batch of beds gives the same bits as each bed alone.
-// The grid barrier spins at most ~0.3 s, then records SEDI_ETIMEOUT and returns;
+// The grid barrier spins at most ~0.8 s, then records SEDI_ETIMEOUT and returns;
 // the other blocks see the record and return at their next barrier.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -146,7 +146,7 @@ __device__ bool grid_barrier(Ctl* ctl, unsigned nblocks, long long spin_limit) {
     } else {
       long long spins = 0;
       while (*gen == g) {
-        if (++spins > spin_limit) {  // ~0.3 s at the default kBarrierSpins
+        if (++spins > spin_limit) {  // ~0.8 s at the default kBarrierSpins
           atomicCAS((int*)&ctl->cg_status, 0, SEDI_ETIMEOUT);
           break;
         }

@@ -213,8 +213,9 @@ struct SmoothBatchDev {
   long long spin_limit;       // polls of a grid-barrier wait before SEDI_ETIMEOUT
 };
 
-// Polls of one grid-barrier wait before the smoother gives up with SEDI_ETIMEOUT
-// (~0.3 s).  A handle may lower it (environment variable SEDI_BARRIER_SPIN_LIMIT,
+// Polls of one wait between blocks before the smoother gives up with SEDI_ETIMEOUT: 192 ns
+// each at the grid barrier, 178 for a tagged word of the resident solver, so ~0.8 s (one SM
+// polling alone; a busy L2 makes it longer).  A handle may lower it (environment variable SEDI_BARRIER_SPIN_LIMIT,
 // read at sedi_create) so that tests can make the wait run out.
 constexpr long long kBarrierSpins = 1ll << 22;
 
