@@ -218,7 +218,9 @@ void sedi_default_params(sedi_params* p);
    variable SEDI_BARRIER_SPIN_LIMIT, read here, lowers the number of polls after
    which a wait between the smoother's thread blocks (meshes too large for one
    thread-block cluster or block) gives up and the averaging returns SEDI_ETIMEOUT (default
-   and most 2^22, about 0.8 s); it exists so tests can make that wait run out. */
+   and most 2^22, about 0.8 s); it exists so tests can make that wait run out.
+   SEDI_SMOOTH_RESIDENT=0, read here too, keeps the handle's meshes off the on-chip
+   smoothing solver, so tests can compare the solvers. */
 int sedi_create(const sedi_params* p, sedi_handle** out);
 void sedi_destroy(sedi_handle* h);
 

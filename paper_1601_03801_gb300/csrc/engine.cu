@@ -33,6 +33,7 @@ struct sedi_handle {
   sedi_params prm{};
   std::string err;
   long long barrier_spins = kBarrierSpins;  // grid-barrier polls before SEDI_ETIMEOUT
+  bool smooth_resident = true;  // meshes may take the on-chip smoothing solver
   cudaStream_t stream = nullptr;
   cudaStream_t side = nullptr;  // capture of conditional bodies
   cudaStream_t own = nullptr;   // default stream of the handle (graphs need a real stream)
@@ -1120,6 +1121,8 @@ int sedi_create(const sedi_params* p, sedi_handle** out) {
     const long long v = std::atoll(lim);
     if (v > 0) h->barrier_spins = std::min(v, kBarrierSpins);
   }
+  // off, for tests that hold the other smoothing solvers to the same results
+  if (const char* on = std::getenv("SEDI_SMOOTH_RESIDENT")) h->smooth_resident = std::atoi(on) != 0;
   fill_params(h);
   const int64_t C = h->P.C;
   h->U.assign(3 * C, 0.0);
@@ -1458,7 +1461,7 @@ static int smooth_dev(sedi_handle* h, int nf, const void* guess, int n_tau = -1,
   int rc = launch_smooth(h->form, h->P, h->phi, guess, nf, h->work, h->st, h->iters_dev,
                          rtol, h->prm.cg_max_iter, n_tau > 0 ? n_tau : h->prm.n_tau,
                          h->prm.tau_scheme, h->coef, h->P.graded ? &h->zs : nullptr,
-                         h->stream, h->barrier_spins);
+                         h->stream, h->barrier_spins, h->smooth_resident);
   if (rc) return fail(h, SEDI_ECUDA, "cooperative launch of the smoother failed: %s", cudaGetErrorString(cudaGetLastError()));
   return 0;
 }
@@ -1958,7 +1961,7 @@ static int ens_average(sedi_handle* h) {
   const double rtol = h->form == FORM_PLAIN ? std::max(h->prm.cg_rtol, 2e-6) : h->prm.cg_rtol;
   if (launch_smooth_batch(h->form, m.data(), B, 7, h->ens_smooth, rtol, h->prm.cg_max_iter,
                           h->prm.n_tau, h->prm.tau_scheme, h->st.ctl, 1 << 30, h->stream,
-                          h->barrier_spins, &h->ens_side))
+                          h->barrier_spins, &h->ens_side, h->smooth_resident))
     return fail(h, SEDI_ECUDA, "cooperative launch of the batched smoother failed: %s",
                 cudaGetErrorString(cudaGetLastError()));
   launch_eps_out_ens(h->form, h->ens, h->stream);

@@ -2093,7 +2093,7 @@ size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme) {
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf, void* work,
                   const DevState& st, int* iters_dev, double rtol, int max_iter, int n_tau,
                   int scheme, const double coef[3], const SmoothZ* z, cudaStream_t s,
-                  long long spin_limit) {
+                  long long spin_limit, bool resident) {
   SmoothMesh m{};
   m.phi = phi;
   m.guess = guess;
@@ -2109,7 +2109,7 @@ int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, in
   if (z) m.z = *z;
   void* batch = (char*)work + align256(smooth_mesh_bytes(form, P.C, nf, scheme));
   return launch_smooth_batch(form, &m, 1, nf, batch, rtol, max_iter, n_tau, scheme, st.ctl,
-                             1 << 30, s, spin_limit);
+                             1 << 30, s, spin_limit, nullptr, resident);
 }
 
 size_t smooth_batch_bytes(int64_t B, int64_t U) {
@@ -2349,7 +2349,8 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
 
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
-                        int max_blocks, cudaStream_t s, long long spin_limit, const SmoothSide* side) {
+                        int max_blocks, cudaStream_t s, long long spin_limit, const SmoothSide* side,
+                        bool resident) {
   if (B < 1 || B > kMaxBeds || nf < 1 || nf > kMaxF || (scheme != TAU_EULER && scheme != TAU_BDF2))
     return -1;
   // every mesh of a batch is graded or none is (one kernel instantiation per launch)
@@ -2376,7 +2377,7 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
     Item it;
     smooth_mesh_layout(form, scheme, meshes[b], &it.m);
     cluster_plan(form, it.m, &it.m.cl_size, &it.m.cl_planes);
-    if (it.m.cl_size == 0 || rs_one_cta(form, it.m)) it.pl = rs_plan(form, it.m, nsm);
+    if (resident && (it.m.cl_size == 0 || rs_one_cta(form, it.m))) it.pl = rs_plan(form, it.m, nsm);
     if (it.m.cl_size > 0 && it.pl.G != 1) {
       mc.push_back(it.m);
     } else if (it.pl.G > 0) {

@@ -240,18 +240,19 @@ int64_t smooth_units(int64_t C);
 size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme);
 size_t smooth_batch_bytes(int64_t B, int64_t U);
 // Smooth every mesh's nf fields in place by n_tau pseudo-steps of the scheme;
-// batch_work: smooth_batch_bytes(B, sum of units) bytes.  Returns 0, -1 (bad sizes)
+// batch_work: smooth_batch_bytes(B, sum of units) bytes.  resident = false keeps every mesh off
+// the resident solver (tests hold the solvers to the same bits).  Returns 0, -1 (bad sizes)
 // or -3 (launch failed).
 int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void* batch_work,
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
                         int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins,
-                        const SmoothSide* side = nullptr);
+                        const SmoothSide* side = nullptr, bool resident = true);
 // Single mesh: work holds smooth_work_bytes(form, C, nf, scheme) = mesh + batch scratch.
 size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme);
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf,
                   void* work, const DevState& st, int* iters_dev, double rtol, int max_iter,
                   int n_tau, int scheme, const double coef[3], const SmoothZ* z,
-                  cudaStream_t s, long long spin_limit = kBarrierSpins);
+                  cudaStream_t s, long long spin_limit = kBarrierSpins, bool resident = true);
 void launch_average_out(int form, const void* phi, const DevParams& P, void* ufe, double* eps,
                         double* Us, double* F, cudaStream_t s);
 void launch_phi_convert(int form, const void* phi, double* out, int64_t n, int to_double,
