@@ -1266,54 +1266,115 @@ __device__ __noinline__ bool rs_receive(N* D, const uint32_t* pull, int nu, int 
   return ok;
 }
 
-// A group's tagged words of the sums: a flag a CTA (its residuals are in place), then the
-// pieces below, each for two parities.
-constexpr int kRsPieces = kThreads;
-static_assert(kClMaxCta <= kRsPieces && kThreads == 256, "");
-__host__ __device__ constexpr size_t rs_sum_words(int G) { return 2 * ((size_t)G + 2 * kRsPieces * kQ); }
-
 // The sums of a round in FP32 words, in the order of the solver that takes this mesh
 // otherwise, so the choice of solver changes no bit of a result (an averaged solid
 // fraction that rounds to another FP32 word would change the drag and a trajectory with it).
-// A piece is what that solver adds in FP64 last: a CTA of its cluster (thread t of 1,024
-// adds columns t, t + 1,024, ..., a warp its threads, the CTA its 32 warps), or for the
-// streaming solver thread t of 256 that adds units t, t + 256, ... of 256 cells.
-// Piece p is formed by CTA p % G from the residuals in global memory and goes to
-// every CTA as tagged words.  This costs two exchanges and a read of the residuals from L2
-// a round: 1,000 of the 5,990 us of seven 128 x 64 x 128 fields, twelve rounds each.
-// ONE: a group of one CTA, its residuals in shared memory.
-template <class T, bool GR, bool ONE>
+
+// A mesh of one CTA, which the cluster solver would hold in one too: thread t of its 1,024
+// adds columns t, t + 1,024, ..., a warp its threads, the CTA its 32 warps in FP64.  The
+// residuals are in shared memory.
+template <class T, bool GR>
+__device__ __forceinline__ void rs_sums_one(const SmoothMeshDev& md, const float* r, const T* b, bool first, float* sl,
+                                         double* tot) {
+  using W = Wide<T>;
+  constexpr int TH = kRsThreads;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nxy = md.nc[0] * md.nc[1], nz = md.nc[2];
+  __syncthreads();
+#pragma unroll 1
+  for (int t = tid; t < kClThreads; t += TH) {
+    float v[kQ] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int s = t; s < nxy; s += kClThreads) {
+      constexpr int kAhead = 8;  // planes whose loads are under way together
+      for (int za = 0; za < nz; za += kAhead) {
+        float rn[kAhead];
+        T bv[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+          const int64_t c = (int64_t)(za + k) * nxy + s;
+          rn[k] = za + k < nz ? r[c] : 0.0f;
+          bv[k] = W::zero();
+          if (first) bv[k] = za + k < nz ? W::ld(b + c) : W::zero();
+        }
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+          if (za + k >= nz) continue;
+          v[0] += rn[k] * rn[k];
+          v[1] += rn[k];
+          if constexpr (GR) v[3] += (float)md.z.w[za + k] * rn[k];
+          const float bn = W::narrow(bv[k]);
+          v[2] += bn * bn;
+        }
+      }
+    }
+    // a butterfly from 16 down for each value: 0 and 2 in the lower half of the lanes, 1
+    // and 3 in the upper
+    const bool up = lane & 16;
+    float a = up ? v[1] : v[0], c = up ? v[3] : v[2];
+    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+    if (first || GR) c += __shfl_xor_sync(0xffffffffu, up ? v[2] : v[3], 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (first || GR) c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    if ((lane & 15) == 0) {
+      float* const to = sl + (t >> 5) * kQ;
+      to[up ? 1 : 0] = a;
+      to[up ? 3 : 2] = c;
+    }
+  }
+  __syncthreads();
+  if (tid < kQ) {
+    double t = 0.0;
+    for (int w = 0; w < kClThreads / 32; ++w) t += (double)sl[w * kQ + tid];
+    tot[tid] = t;
+  }
+  __syncthreads();
+}
+
+// A group's tagged words of the sums: a flag a CTA (its residuals are in place), then the
+// pieces below, each for two parities.
+constexpr int kRsPieces = kThreads;
+static_assert(kThreads == 256, "");
+__host__ __device__ constexpr size_t rs_sum_words(int G) { return 2 * ((size_t)G + 2 * kRsPieces * kQ); }
+
+// One CTA: as above.  Several CTAs, a mesh that the streaming solver would take: its thread t of 256
+// adds units t, t + 256, ... of 256 cells in FP64, a piece.  Piece p is formed by CTA p % G
+// from the residuals in global memory and goes to every CTA as tagged words.  This costs two
+// exchanges and a read of the residuals from L2 a round: 1,000 of the 5,990 us of seven
+// 128 x 64 x 128 fields, twelve rounds each.
+template <class T, bool GR>
 __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, const T* b, bool first, int G, int rank,
                                      float* sl, unsigned long long* words, uint32_t seq, double* tot, int* s_ok,
                                      Ctl* ctl, long long spin_limit) {
   using W = Wide<T>;
-  constexpr int TH = kRsThreads, kWarps = TH / 32, kRanks = 10, kUnits = 40;  // 5,120 bytes of sl
+  constexpr int TH = kRsThreads, kWarps = TH / 32, kUnits = 40;  // 5,120 bytes of sl
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int nxy = md.nc[0] * md.nc[1];
   const int64_t C = md.C;
+  if (G == 1) {
+    rs_sums_one<T, GR>(md, r, b, first, sl, tot);
+    return true;
+  }
   unsigned long long* const flags = words + (size_t)(seq & 1) * G;
   unsigned long long* const pieces = words + 2 * (size_t)G + (size_t)(seq & 1) * 2 * kRsPieces * kQ;
   __syncthreads();
-  if (!ONE) {
-    if (tid == 0) {
-      __threadfence();
-      put1(flags + rank, 0u, seq);
-    }
-    if (tid < G) {
-      Spin spin;
-      while ((uint32_t)(get1(flags + tid) >> 32) != seq)
-        if (!spin.go(ctl, spin_limit)) {
-          *s_ok = 0;
-          break;
-        }
-      __threadfence();
-    }
-    __syncthreads();
-    if (!*s_ok) return false;
+  if (tid == 0) {
+    __threadfence();
+    put1(flags + rank, 0u, seq);
   }
-  auto put_piece = [&](int p, int q, double v) {
-    put2(pieces + ((size_t)p * kQ + q) * 2, as_word(v, 0), as_word(v, 1), seq);
-  };
+  if (tid < G) {
+    Spin spin;
+    while ((uint32_t)(get1(flags + tid) >> 32) != seq)
+      if (!spin.go(ctl, spin_limit)) {
+        *s_ok = 0;
+        break;
+      }
+    __threadfence();
+  }
+  __syncthreads();
+  if (!*s_ok) return false;
   bool ok = true;
   auto get_piece = [&](int p, int q) {
     const unsigned long long* const at = pieces + ((size_t)p * kQ + q) * 2;
@@ -1327,23 +1388,6 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
     double d;
     of_words(d, (uint32_t)v.a, (uint32_t)v.b);
     return d;
-  };
-  // warp sums of four values, a butterfly from 16 down for each: q0 and q2 in the lower
-  // half of the lanes, q1 and q3 in the upper
-  auto warp_sums = [&](float (&v)[kQ], float* to, int stride) {
-    const bool up = lane & 16;
-    float a = up ? v[1] : v[0], c = up ? v[3] : v[2];
-    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
-    if (first || GR) c += __shfl_xor_sync(0xffffffffu, up ? v[2] : v[3], 16);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (first || GR) c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if ((lane & 15) == 0) {
-      to[(up ? 1 : 0) * stride] = a;
-      to[(up ? 3 : 2) * stride] = c;
-    }
   };
   // warp sums of the 8 warps of a unit, two values each: the same butterflies as a
   // reduce-scatter, a lane keeps half of its sums at every step
@@ -1364,148 +1408,78 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
     a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
     if (!(lane & 1)) to[lane >> 1] = a[0];  // [value][warp]
   };
-  auto load = [&](int64_t c) {
-    if constexpr (ONE) return r[c];
-    else return __ldcg(r + c);
-  };
-  if (md.cl_size > 0) {
-    const int cs = md.cl_size, P = md.cl_planes;
-    if (tid < kQ && ONE) tot[tid] = 0.0;
-    for (int r0 = rank; r0 < cs; r0 += kRanks * G) {
-      for (int i = 0; i < kRanks && r0 + i * G < cs; ++i) {
-        const int z0 = (r0 + i * G) * P, z1 = z0 + P < md.nc[2] ? z0 + P : md.nc[2];
+  const int nu = (int)md.nu, np = nu < kRsPieces ? nu : kRsPieces;
+  const int mine = rank < np ? (np - rank + G - 1) / G : 0;  // this CTA's pieces rank, rank + G, ...
+  const int all = mine * ((nu + kRsPieces - 1) / kRsPieces);
+  double acc = 0.0;  // of piece tid / kQ of them (128 at most), sum tid % kQ
+  for (int i0 = 0; i0 < all; i0 += kUnits) {  // units in order for every piece
+    const int n = all - i0 < kUnits ? all - i0 : kUnits;
 #pragma unroll 1
-        for (int t = tid; t < kClThreads; t += TH) {
-          float v[kQ] = {0.0f, 0.0f, 0.0f, 0.0f};
-          for (int s = t; s < nxy; s += kClThreads) {
-            constexpr int kAhead = 8;  // planes whose loads are under way together
-            for (int za = z0; za < z1; za += kAhead) {
-              float rn[kAhead];
-              T bv[kAhead];
+    for (int s = wid; s < n; s += kWarps) {  // a warp takes the 8 warps of a unit
+      const int i = i0 + s, u = rank + i % mine * G + i / mine * kRsPieces;
+      const int64_t c0 = (int64_t)u * kThreads + lane;
+      float rn[8], v[2][8];
+      T bv[8];
 #pragma unroll
-              for (int k = 0; k < kAhead; ++k) {
-                const int64_t c = (int64_t)(za + k) * nxy + s;
-                rn[k] = za + k < z1 ? load(c) : 0.0f;
-                bv[k] = W::zero();
-                if (first) bv[k] = za + k < z1 ? W::ld(b + c) : W::zero();
-              }
+      for (int w = 0; w < 8; ++w) {  // every load before the first use
+        const int64_t c = c0 + w * 32;
+        const bool in = u < nu && c < C;
+        rn[w] = in ? __ldcg(r + c) : 0.0f;
+        bv[w] = W::zero();
+        if (first) bv[w] = in ? W::ld(b + c) : W::zero();
+      }
 #pragma unroll
-              for (int k = 0; k < kAhead; ++k) {
-                if (za + k >= z1) continue;
-                v[0] += rn[k] * rn[k];
-                v[1] += rn[k];
-                if constexpr (GR) v[3] += (float)md.z.w[za + k] * rn[k];
-                const float bn = W::narrow(bv[k]);
-                v[2] += bn * bn;
-              }
-            }
-          }
-          warp_sums(v, sl + (i * 32 + (t >> 5)) * kQ, 1);
-        }
+      for (int w = 0; w < 8; ++w) {
+        v[0][w] = rn[w] * rn[w];
+        v[1][w] = rn[w];
       }
-      __syncthreads();
-      const int q = tid % kQ;
-      for (int i = ONE ? 0 : tid / kQ; i < kRanks && r0 + i * G < cs && tid < (ONE ? kQ : kRanks * kQ); ++i) {
-        double t = 0.0;
-        for (int w = 0; w < 32; ++w) t += (double)sl[(i * 32 + w) * kQ + q];
-        if (ONE) {
-          tot[q] += t;
-        } else {
-          put_piece(r0 + i * G, q, t);
-          break;
-        }
-      }
-      __syncthreads();
-    }
-    if (!ONE) {
-      double* const part = (double*)sl;
-      for (int k = tid; k < cs * kQ; k += TH) part[k] = get_piece(k / kQ, k % kQ);
-      if (!ok) *s_ok = 0;
-      __syncthreads();
-      if (tid < kQ) {
-        double t = 0.0;
-        for (int k = 0; k < cs; ++k) t += part[k * kQ + tid];
-        tot[tid] = t;
-      }
-    }
-  } else {
-    const int nu = (int)md.nu, np = nu < kRsPieces ? nu : kRsPieces;
-    const int mine = rank < np ? (np - rank + G - 1) / G : 0;  // this CTA's pieces rank, rank + G, ...
-    const int all = mine * ((nu + kRsPieces - 1) / kRsPieces);
-    double acc = 0.0;  // of piece tid / kQ of them (128 at most), sum tid % kQ
-    for (int i0 = 0; i0 < all; i0 += kUnits) {  // units in order for every piece
-      const int n = all - i0 < kUnits ? all - i0 : kUnits;
-#pragma unroll 1
-      for (int s = wid; s < n; s += kWarps) {  // a warp takes the 8 warps of a unit
-        const int i = i0 + s, u = rank + i % mine * G + i / mine * kRsPieces;
-        const int64_t c0 = (int64_t)u * kThreads + lane;
-        float rn[8], v[2][8];
-        T bv[8];
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {  // every load before the first use
-          const int64_t c = c0 + w * 32;
-          const bool in = u < nu && c < C;
-          rn[w] = in ? load(c) : 0.0f;
-          bv[w] = W::zero();
-          if (first) bv[w] = in ? W::ld(b + c) : W::zero();
-        }
+      unit_warps(v, sl + s * (8 * kQ));
+      if (GR || first) {
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-          v[0][w] = rn[w] * rn[w];
-          v[1][w] = rn[w];
-        }
-        unit_warps(v, sl + s * (8 * kQ));
-        if (GR || first) {
-#pragma unroll
-          for (int w = 0; w < 8; ++w) {
-            const float bn = W::narrow(bv[w]);
-            v[0][w] = bn * bn;
-            v[1][w] = 0.0f;
-            if constexpr (GR) {
-              const int c = (int)c0 + w * 32;
-              if (u < nu && c < C) v[1][w] = (float)md.z.w[c / nxy] * rn[w];
-            }
+          const float bn = W::narrow(bv[w]);
+          v[0][w] = bn * bn;
+          v[1][w] = 0.0f;
+          if constexpr (GR) {
+            const int c = (int)c0 + w * 32;
+            if (u < nu && c < C) v[1][w] = (float)md.z.w[c / nxy] * rn[w];
           }
-          unit_warps(v, sl + s * (8 * kQ) + 16);
         }
+        unit_warps(v, sl + s * (8 * kQ) + 16);
       }
-      __syncthreads();
-      if (tid < n * kQ && (GR || first || tid % kQ < 2)) {  // a unit's sum, in the place of its warps'
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) t += (double)sl[tid * 8 + w];
-        ((double*)sl)[tid * 4] = t;
-      }
-      __syncthreads();
-      if (tid < mine * kQ) {
-        const int j = tid / kQ, q = tid % kQ;
-        for (int k = ((j - i0) % mine + mine) % mine; k < n; k += mine)
-          if (rank + j * G + (i0 + k) / mine * kRsPieces < nu) acc += ((double*)sl)[(k * kQ + q) * 4];
-      }
-      __syncthreads();
-    }
-    double* const own = (double*)sl;       // one CTA: the pieces
-    double* const ws = (double*)sl + 600;  // sums of 32 pieces
-    if (tid < mine * kQ) {
-      if (!ONE) put_piece(rank + tid / kQ * G, tid % kQ, acc);
-      else own[tid] = acc;
     }
     __syncthreads();
-#pragma unroll
-    for (int k = wid; k < 8 * kQ; k += kWarps) {
-      const int p = k / kQ * 32 + lane, q = k % kQ;
-      double v = p < np ? (!ONE ? get_piece(p, q) : own[p * kQ + q]) : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) ws[k] = v;
-    }
-    if (!ok) *s_ok = 0;
-    __syncthreads();
-    if (tid < kQ) {
+    if (tid < n * kQ && (GR || first || tid % kQ < 2)) {  // a unit's sum, in the place of its warps'
       double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += ws[w * kQ + tid];
-      tot[tid] = t;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t += (double)sl[tid * 8 + w];
+      ((double*)sl)[tid * 4] = t;
     }
+    __syncthreads();
+    if (tid < mine * kQ) {
+      const int j = tid / kQ, q = tid % kQ;
+      for (int k = ((j - i0) % mine + mine) % mine; k < n; k += mine)
+        if (rank + j * G + (i0 + k) / mine * kRsPieces < nu) acc += ((double*)sl)[(k * kQ + q) * 4];
+    }
+    __syncthreads();
+  }
+  double* const ws = (double*)sl;  // sums of 32 pieces
+  if (tid < mine * kQ)
+    put2(pieces + ((size_t)(rank + tid / kQ * G) * kQ + tid % kQ) * 2, as_word(acc, 0), as_word(acc, 1), seq);
+#pragma unroll
+  for (int k = wid; k < 8 * kQ; k += kWarps) {
+    const int p = k / kQ * 32 + lane, q = k % kQ;
+    double v = p < np ? get_piece(p, q) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) ws[k] = v;
+  }
+  if (!ok) *s_ok = 0;
+  __syncthreads();
+  if (tid < kQ) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += ws[w * kQ + tid];
+    tot[tid] = t;
   }
   __syncthreads();
   return *s_ok;
@@ -1834,11 +1808,9 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
         }
         ++rseq;
         if constexpr (kOrder) {
-          auto sums = [&](auto one) {
-            return rs_sums<T, GR, decltype(one)::value>(md, (const float*)s_g.r, s_g.b, round == 0, G, rank, (float*)s_part,
-                                                        s_g.sums, rseq, s_tot, &s_ok, a.ctl, a.spin_limit);
-          };
-          if (!(G == 1 ? sums(std::true_type{}) : sums(std::false_type{}))) return;
+          if (!rs_sums<T, GR>(md, (const float*)s_g.r, s_g.b, round == 0, G, rank, (float*)s_part, s_g.sums, rseq, s_tot,
+                              &s_ok, a.ctl, a.spin_limit))
+            return;
         } else {
           // ---- the group's sums: warp, CTA, then the CTAs in rank order
 #pragma unroll
