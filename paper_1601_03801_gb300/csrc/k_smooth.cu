@@ -1041,8 +1041,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
 // CTA (ix, iy, iz) of the group holds a brick of bx x by x bz cells.
 // x (wide) and the recursive residual q live in registers (a thread owns chunks of
 // kRsZ cells along z), the direction d in shared memory, double-buffered, with halos.
-// Same iteration as the solvers above, operation for operation; in FP32 words the sums of a
-// round are theirs too (rs_sums), so are all bits of a result.
+// Same iteration as the solvers above, operation for operation; the sums of a round are theirs
+// too (rs_sums), so are all bits of a result.
 // Halos between CTAs go through global memory (they stay in L2) as 8-byte words of a value
 // and the exchange's number, so a receiver polls the data itself: no fence, no flag and no
 // barrier between a store and its use.  A round's sums travel the same way.  Every wait is
@@ -1068,6 +1068,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
 // streaming solver ran it on 35 blocks).
 constexpr int kRsZ = 4;              // cells of a chunk
 constexpr int kRsMaxGroup = 160;     // CTAs of a group at most
+constexpr int kRsSumBytes = 5120;    // shared memory of a round's sums
 constexpr size_t kRsSmem = 176 * 1024;  // dynamic shared memory of a CTA at most
 
 // Threads of a CTA, and the chunks a thread holds at most: their x and q are 12 registers
@@ -1266,11 +1267,11 @@ __device__ __noinline__ bool rs_receive(N* D, const uint32_t* pull, int nu, int 
   return ok;
 }
 
-// The sums of a round in FP32 words, in the order of the solver that takes this mesh
-// otherwise, so the choice of solver changes no bit of a result (an averaged solid
-// fraction that rounds to another FP32 word would change the drag and a trajectory with it).
+// The sums of a round, in the order of the solver that takes this mesh otherwise, so neither the
+// choice of solver nor a cut changes a bit of a result (an averaged solid fraction that
+// rounds to another FP32 word would change the drag and a trajectory with it).
 
-// A mesh of one CTA, which the cluster solver would hold in one too: thread t of its 1,024
+// A mesh of one CTA (FP32 words), which the cluster solver would hold in one too: thread t of its 1,024
 // adds columns t, t + 1,024, ..., a warp its threads, the CTA its 32 warps in FP64.  The
 // residuals are in shared memory.
 template <class T, bool GR>
@@ -1345,17 +1346,20 @@ __host__ __device__ constexpr size_t rs_sum_words(int G) { return 2 * ((size_t)G
 // exchanges and a read of the residuals from L2 a round: 1,000 of the 5,990 us of seven
 // 128 x 64 x 128 fields, twelve rounds each.
 template <class T, bool GR>
-__device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, const T* b, bool first, int G, int rank,
-                                     float* sl, unsigned long long* words, uint32_t seq, double* tot, int* s_ok,
+__device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const typename Wide<T>::N* r, const T* b, bool first,
+                                     int G, int rank, typename Wide<T>::N* sl, unsigned long long* words, uint32_t seq, double* tot, int* s_ok,
                                      Ctl* ctl, long long spin_limit) {
   using W = Wide<T>;
-  constexpr int TH = kRsThreads, kWarps = TH / 32, kUnits = 40;  // 5,120 bytes of sl
+  using N = typename W::N;
+  constexpr int TH = kRsThreads, kWarps = TH / 32, kUnits = kRsSumBytes / (8 * kQ * sizeof(N));
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int nxy = md.nc[0] * md.nc[1];
   const int64_t C = md.C;
-  if (G == 1) {
-    rs_sums_one<T, GR>(md, r, b, first, sl, tot);
-    return true;
+  if constexpr (sizeof(N) == 4) {
+    if (G == 1) {
+      rs_sums_one<T, GR>(md, r, b, first, sl, tot);
+      return true;
+    }
   }
   unsigned long long* const flags = words + (size_t)(seq & 1) * G;
   unsigned long long* const pieces = words + 2 * (size_t)G + (size_t)(seq & 1) * 2 * kRsPieces * kQ;
@@ -1391,8 +1395,8 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
   };
   // warp sums of the 8 warps of a unit, two values each: the same butterflies as a
   // reduce-scatter, a lane keeps half of its sums at every step
-  auto unit_warps = [&](float (&v)[2][8], float* to) {
-    float a[8];
+  auto unit_warps = [&](N (&v)[2][8], N* to) {
+    N a[8];
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
       const bool up = lane & 16;
@@ -1418,13 +1422,13 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
     for (int s = wid; s < n; s += kWarps) {  // a warp takes the 8 warps of a unit
       const int i = i0 + s, u = rank + i % mine * G + i / mine * kRsPieces;
       const int64_t c0 = (int64_t)u * kThreads + lane;
-      float rn[8], v[2][8];
+      N rn[8], v[2][8];
       T bv[8];
 #pragma unroll
       for (int w = 0; w < 8; ++w) {  // every load before the first use
         const int64_t c = c0 + w * 32;
         const bool in = u < nu && c < C;
-        rn[w] = in ? __ldcg(r + c) : 0.0f;
+        rn[w] = in ? __ldcg(r + c) : N(0);
         bv[w] = W::zero();
         if (first) bv[w] = in ? W::ld(b + c) : W::zero();
       }
@@ -1437,12 +1441,12 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
       if (GR || first) {
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-          const float bn = W::narrow(bv[w]);
+          const N bn = W::narrow(bv[w]);
           v[0][w] = bn * bn;
-          v[1][w] = 0.0f;
+          v[1][w] = N(0);
           if constexpr (GR) {
             const int c = (int)c0 + w * 32;
-            if (u < nu && c < C) v[1][w] = (float)md.z.w[c / nxy] * rn[w];
+            if (u < nu && c < C) v[1][w] = (N)md.z.w[c / nxy] * rn[w];
           }
         }
         unit_warps(v, sl + s * (8 * kQ) + 16);
@@ -1453,13 +1457,13 @@ __device__ __noinline__ bool rs_sums(const SmoothMeshDev& md, const float* r, co
       double t = 0.0;
 #pragma unroll
       for (int w = 0; w < 8; ++w) t += (double)sl[tid * 8 + w];
-      ((double*)sl)[tid * 4] = t;
+      ((double*)sl)[tid * sizeof(N)] = t;
     }
     __syncthreads();
     if (tid < mine * kQ) {
       const int j = tid / kQ, q = tid % kQ;
       for (int k = ((j - i0) % mine + mine) % mine; k < n; k += mine)
-        if (rank + j * G + (i0 + k) / mine * kRsPieces < nu) acc += ((double*)sl)[(k * kQ + q) * 4];
+        if (rank + j * G + (i0 + k) / mine * kRsPieces < nu) acc += ((double*)sl)[(k * kQ + q) * sizeof(N)];
     }
     __syncthreads();
   }
@@ -1490,15 +1494,13 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
   using W = Wide<T>;
   using N = typename W::N;
   using P = Pub<T>;
-  constexpr bool kOrder = sizeof(N) == 4;  // sums in the other solvers' order (rs_sums)
-  constexpr int TH = kRsThreads, kWarps = TH / 32;
+  constexpr int TH = kRsThreads;
   constexpr int NW = sizeof(N) / 4;  // 32-bit words of a narrow value
   // a chunk's first word: index of its first cell, valid cells, chunk along z; its second
   // word: the indexes of the cells below and above it
   constexpr int kCnt = 18, kZc = 21;
   extern __shared__ __align__(16) unsigned char s_dyn[];
-  __shared__ double s_part[kRsMaxGroup][kQ];  // every CTA's sums
-  __shared__ double s_red[kOrder ? 1 : kWarps][kQ];
+  __shared__ double s_part[kRsSumBytes / 8];  // rs_sums
   __shared__ double s_tot[kQ], s_shift;
   __shared__ uint2 s_info[M * TH];
   __shared__ int s_cell[M * TH];  // first cell of a chunk in the mesh
@@ -1513,10 +1515,9 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
     N* r;                  // the narrow true residual between its pass and the step loop (FP32
                            // words in one CTA: in shared memory)
     unsigned long long* halo;  // grid: the group's tagged halo words, [CTA][parity][channel][hw]
-    unsigned long long* sums;  // grid: the group's tagged words of the sums (rs_sums; in
-                               // FP64 [parity][CTA][kQ][2])
+    unsigned long long* sums;  // grid: the group's tagged words of the sums (rs_sums)
   } s_g;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x;
   const int G = a.rs_G, rank = (int)(blockIdx.x % (unsigned)G);
   const int64_t grp = blockIdx.x / (unsigned)G, ngrp = gridDim.x / (unsigned)G;
   uint32_t seq = 0, rseq = 0;  // halo exchanges and reductions so far
@@ -1584,7 +1585,7 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
       s_g.b = (T*)md.b + f * C;
       s_g.xp = md.xp ? (T*)md.xp + f * C : nullptr;
       s_g.guess = md.guess ? (const T*)md.guess + f * C : nullptr;
-      s_g.r = kOrder && G == 1 ? (N*)(s_pull + nu_max) : (N*)md.q + f * C;
+      s_g.r = G == 1 ? (N*)(s_pull + nu_max) : (N*)md.q + f * C;
       s_g.sums = (unsigned long long*)md.d[0] + (size_t)grp * rs_sum_words(G);
       s_g.halo = (unsigned long long*)md.d[0] + (size_t)ngrp * rs_sum_words(G) + (size_t)grp * G * 2 * P::n * hw * NW;
     }
@@ -1745,9 +1746,8 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
           }
         }
         if (!exchange(0, P::n)) return;
-        // ---- true residual (wide), its narrow copy to global memory, in FP64 the sums; the
-        //      next chunk's b is loaded ahead
-        [[maybe_unused]] N sum[kQ] = {};
+        // ---- true residual (wide), its narrow copy to global memory; the next chunk's b is
+        //      loaded ahead
         {
           const T cf[3] = {coef_w<T>(sp, 0), coef_w<T>(sp, 1), coef_w<T>(sp, 2)};
           T bn[kRsZ];
@@ -1785,15 +1785,6 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
                 else
                   rn = Resid<T>::eval(cf, c[z], l[z], r[z], fr[z], bk[z], below, above, bv[z]);
                 out(z, rn);
-                if constexpr (!kOrder) {
-                  sum[0] += rn * rn;
-                  sum[1] += rn;
-                  if constexpr (GR) sum[3] += (N)md.z.w[kz + z] * rn;
-                  if (round == 0) {
-                    const N b1 = W::narrow(bv[z]);
-                    sum[2] += b1 * b1;
-                  }
-                }
               }
               below = c[z];
             }
@@ -1807,93 +1798,46 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
           }
         }
         ++rseq;
-        if constexpr (kOrder) {
-          if (!rs_sums<T, GR>(md, (const float*)s_g.r, s_g.b, round == 0, G, rank, (float*)s_part, s_g.sums, rseq, s_tot,
-                              &s_ok, a.ctl, a.spin_limit))
-            return;
-        } else {
-          // ---- the group's sums: warp, CTA, then the CTAs in rank order
-#pragma unroll
-          for (int q = 0; q < kQ; ++q) {
-            double t = sum[q];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) s_red[wid][q] = t;
+        if (!rs_sums<T, GR>(md, s_g.r, s_g.b, round == 0, G, rank, (N*)s_part, s_g.sums, rseq, s_tot, &s_ok, a.ctl,
+                            a.spin_limit))
+          return;
+        // one thread of every CTA decides: every CTA takes the same decision
+        if (tid == 0) {
+          const double rr = s_tot[0], sr = s_tot[1];
+          if (round == 0) bb = s_tot[2];
+          const int zero = !(bb > 0.0);
+          double shift, rrp;
+          if (GR) {
+            // the shift keeps sum(w x) = sum(w b); |r - s|^2 = |r|^2 - 2 s sum r + C s^2
+            shift = zero ? 0.0 : s_tot[3] / md.z.wsum;
+            rrp = fmax(rr - 2.0 * shift * sr + (double)C * shift * shift, 0.0);
+          } else {
+            shift = zero ? 0.0 : sr / (double)C;
+            rrp = fmax(rr - sr * sr / (double)C, 0.0);
           }
-          __syncthreads();
-          if (tid < kQ) {
-            double t = 0.0;
-            for (int r = 0; r < kWarps; ++r) t += s_red[r][tid];
-            s_tot[tid] = t;
-            if (G > 1)
-              put2(s_g.sums + (((size_t)(rseq & 1) * G + rank) * kQ + tid) * 2, as_word(t, 0), as_word(t, 1), rseq);
-          }
-          if (G > 1) {
-            bool ok = true;
-            for (int t = tid; t < G * kQ; t += TH) {
-              const unsigned long long* p = s_g.sums + ((size_t)(rseq & 1) * G * kQ + t) * 2;
-              Tag2 v;
-              v.load(p);
-              Spin spin;
-              while (!v.is(rseq) && ok) {
-                ok = spin.go(a.ctl, a.spin_limit);
-                v.load(p);
-              }
-              of_words(s_part[t / kQ][t % kQ], (uint32_t)v.a, (uint32_t)v.b);
-            }
-            if (!ok) s_ok = 0;
-            __syncthreads();
-            if (!s_ok) return;
-          }
-        }
-        // the first warp of every CTA sums and decides: every CTA takes the same decision
-        if (wid == 0) {
-          if (!kOrder && G > 1) {
-            const int q = lane >> 3;
-            double t = 0.0;
-            for (int r = lane & 7; r < G; r += 8) t += s_part[r][q];
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if ((lane & 7) == 0) s_tot[q] = t;
-            __syncwarp();
-          }
-          if (lane == 0) {
-            const double rr = s_tot[0], sr = s_tot[1];
-            if (round == 0) bb = s_tot[2];
-            const int zero = !(bb > 0.0);
-            double shift, rrp;
-            if (GR) {
-              // the shift keeps sum(w x) = sum(w b); |r - s|^2 = |r|^2 - 2 s sum r + C s^2
-              shift = zero ? 0.0 : s_tot[3] / md.z.wsum;
-              rrp = fmax(rr - 2.0 * shift * sr + (double)C * shift * shift, 0.0);
+          int k = 0;
+          if (!zero && !(rrp <= a.rtol2 * bb)) {
+            // |r_k| <= 2 sig^k |r_0|: enough steps for the tolerance, or for the reduction
+            // the narrow word can deliver in one round (as the cluster solver forms the
+            // count where it would take the mesh, else as the streaming one)
+            if (md.cl_size > 0) {
+              const float need = fmaxf(0.5f * sqrtf((float)(a.rtol2 * bb / rrp)), (float)W::kFloor);
+              k = sp.sig > 0.0 ? (int)ceilf(logf(need) / logf((float)sp.sig)) : 1;
             } else {
-              shift = zero ? 0.0 : sr / (double)C;
-              rrp = fmax(rr - sr * sr / (double)C, 0.0);
+              const double need = fmax(0.5 * sqrt(a.rtol2 * bb / rrp), W::kFloor);
+              k = sp.sig > 0.0 ? (int)ceil(log(need) / log(sp.sig)) : 1;
             }
-            int k = 0;
-            if (!zero && !(rrp <= a.rtol2 * bb)) {
-              // |r_k| <= 2 sig^k |r_0|: enough steps for the tolerance, or for the reduction
-              // the narrow word can deliver in one round (as the cluster solver forms the
-              // count where it would take the mesh, else as the streaming one)
-              if (md.cl_size > 0) {
-                const float need = fmaxf(0.5f * sqrtf((float)(a.rtol2 * bb / rrp)), (float)W::kFloor);
-                k = sp.sig > 0.0 ? (int)ceilf(logf(need) / logf((float)sp.sig)) : 1;
-              } else {
-                const double need = fmax(0.5 * sqrt(a.rtol2 * bb / rrp), W::kFloor);
-                k = sp.sig > 0.0 ? (int)ceil(log(need) / log(sp.sig)) : 1;
-              }
-              if (k < 1) k = 1;
-              if (k > kMaxStepsRound) k = kMaxStepsRound;
-              if (total + k > a.max_iter) k = a.max_iter - total;
-              if (k <= 0) {
-                k = 0;
-                if (rank == 0) atomicCAS((int*)&a.ctl->cg_status, 0, SEDI_EDIVERGED);
-              }
+            if (k < 1) k = 1;
+            if (k > kMaxStepsRound) k = kMaxStepsRound;
+            if (total + k > a.max_iter) k = a.max_iter - total;
+            if (k <= 0) {
+              k = 0;
+              if (rank == 0) atomicCAS((int*)&a.ctl->cg_status, 0, SEDI_EDIVERGED);
             }
-            s_k = k;
-            s_shift = shift;
-            s_zero = zero;
           }
+          s_k = k;
+          s_shift = shift;
+          s_zero = zero;
         }
         __syncthreads();
         const int k = s_k, zero = s_zero;
@@ -2211,7 +2155,7 @@ void cluster_plan(int form, const SmoothMeshDev& m, int* csize, int* planes) {
 
 // How the resident solver cuts a mesh into px x py x pz bricks (G CTAs), or G = 0 when no
 // cut fits.  The choice depends on the mesh, the form and the device alone, so a mesh is
-// smoothed with the same bits in any batch.
+// planned the same way in any batch; no bit of a result depends on it.
 struct RsPlan {
   int G = 0, px = 0, py = 0, pz = 0, groups = 0;
   int chunks = 0;             // of a thread
@@ -2337,8 +2281,7 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
   // 440 us in a cluster solver's CTA, 250 here), larger meshes that fit a cluster's shared
   // memory the cluster solver (one launch for every mesh of a cluster size), still larger
   // ones the resident solver again where a cut of the whole chip fits, else the streaming grid
-  // solver.  In FP64 there is no cluster solver.  The choice depends on the mesh alone, and
-  // in FP32 words no bit of a result depends on it.
+  // solver.  In FP64 there is no cluster solver.  No bit of a result depends on the choice.
   struct Item {
     SmoothMeshDev m;
     RsPlan pl;

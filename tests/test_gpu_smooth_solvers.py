@@ -84,3 +84,20 @@ def test_streaming_barrier_timeout_is_reported_and_handle_recovers(monkeypatch):
     g.sync()
     out, _ = sedi.Sedi(dict(prm, precision_form="split")).smooth(phi)
     np.testing.assert_array_equal(out, want)
+
+
+# whole-chip groups from one cell a brick up, cuts that change with the number of fields, and
+# meshes of one cell across
+@pytest.mark.parametrize("ncell,periodic,scheme,grading", [
+    ((5, 7, 9), (1, 0, 1), 1, 1.0), ((8, 8, 8), (1, 1, 0), 0, 1.0), ((13, 17, 6), (0, 0, 0), 1, 3.0),
+    ((19, 15, 31), (1, 1, 0), 0, 1.0), ((70, 2, 3), (1, 1, 1), 0, 1.0), ((3, 1, 41), (0, 1, 0), 0, 1.0),
+    ((37, 41, 45), (1, 1, 0), 1, 2.0), ((53, 51, 49), (1, 1, 1), 0, 1.0), ((100, 100, 1), (0, 1, 0), 1, 1.0)])
+def test_same_fp64_bits_from_every_solver_and_cut(monkeypatch, ncell, periodic, scheme, grading):
+    on, off = handles(monkeypatch, mesh(ncell, periodic, scheme, grading), "fp64")
+    phi = random_fields(ncell, 8, seed=19)
+    phi[2] = 0.0
+    want, steps = off.smooth(phi)
+    for nf in (8, 7, 2, 1):
+        out, it = on.smooth(phi[:nf])
+        np.testing.assert_array_equal(out, want[:nf])
+        np.testing.assert_array_equal(it, steps[:nf])
