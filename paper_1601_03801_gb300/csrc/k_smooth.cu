@@ -2154,8 +2154,7 @@ void cluster_plan(int form, const SmoothMeshDev& m, int* csize, int* planes) {
 }
 
 // How the resident solver cuts a mesh into px x py x pz bricks (G CTAs), or G = 0 when no
-// cut fits.  The choice depends on the mesh, the form and the device alone, so a mesh is
-// planned the same way in any batch; no bit of a result depends on it.
+// cut fits, for nf fields.  No bit of a result depends on the cut.
 struct RsPlan {
   int G = 0, px = 0, py = 0, pz = 0, groups = 0;
   int chunks = 0;             // of a thread
@@ -2173,7 +2172,7 @@ bool rs_one_cta(int form, const SmoothMeshDev& m) {
          (int64_t)m.nc[0] * m.nc[1] * ((m.nc[2] + kRsZ - 1) / kRsZ) <= kRsThreads * kRsChunks;
 }
 
-RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
+RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
   const size_t word = form == FORM_FP64 ? 8 : 4;
   const int nx = m.nc[0], ny = m.nc[1], nz = m.nc[2];
   const int T = kRsThreads, top = T * (word == 8 ? kRsChunks : kRsChunksBig);
@@ -2206,7 +2205,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
       if ((int64_t)rs_tag_bytes(G, halo) * groups > m.halo_bytes) return;
       t += 1.5 + 0.0018 * units + 0.00015 * planes;
     }
-    const double cost = t * ((7 + groups - 1) / groups);  // waves of the averaging's seven fields
+    const double cost = t * ((nf + groups - 1) / groups);  // waves of the fields
     if (cost < best_cost) {
       best_cost = cost;
       best.G = G;
@@ -2224,7 +2223,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nsm) {
     if (best.G) return best;
   }
   // for every number of groups at once, the largest groups
-  for (int g = 1; g <= 7; ++g) {
+  for (int g = 1; g <= nf; ++g) {
     const int gmax = nsm / g < kRsMaxGroup ? nsm / g : kRsMaxGroup;
     for (int pz = 1; pz <= 40 && pz <= gmax; ++pz)
       for (int py = 1; py * pz <= gmax; ++py) consider(gmax / (py * pz), py, pz, g);
@@ -2248,14 +2247,13 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
   }
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRsThreads, pl.smem) != cudaSuccess) return -3;
-  const int groups = pl.groups < a.nf ? pl.groups : a.nf;
-  if ((int64_t)per_sm * nsm < (int64_t)groups * pl.G) return -3;
+  if ((int64_t)per_sm * nsm < (int64_t)pl.groups * pl.G) return -3;
   // no tagged word of an earlier launch may pass for this one's: exchanges count from 1
-  const size_t bytes = rs_tag_bytes(pl.G, pl.halo) * groups;
+  const size_t bytes = rs_tag_bytes(pl.G, pl.halo) * pl.groups;
   if (cudaMemsetAsync(m.d[0], 0, bytes, s) != cudaSuccess) return -3;
   SmoothBatchDev args = a;
   void* p[] = {&args};
-  return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)(groups * pl.G)), dim3(kRsThreads), p, pl.smem, s) ==
+  return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)(pl.groups * pl.G)), dim3(kRsThreads), p, pl.smem, s) ==
                  cudaSuccess
              ? 0
              : -3;
@@ -2292,7 +2290,7 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
     Item it;
     smooth_mesh_layout(form, scheme, meshes[b], &it.m);
     cluster_plan(form, it.m, &it.m.cl_size, &it.m.cl_planes);
-    if (resident && (it.m.cl_size == 0 || rs_one_cta(form, it.m))) it.pl = rs_plan(form, it.m, nsm);
+    if (resident && (it.m.cl_size == 0 || rs_one_cta(form, it.m))) it.pl = rs_plan(form, it.m, nf, nsm);
     if (it.m.cl_size > 0 && it.pl.G != 1) {
       mc.push_back(it.m);
     } else if (it.pl.G > 0) {

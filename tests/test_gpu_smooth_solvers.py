@@ -2,6 +2,8 @@
 of them takes a mesh: the on-chip solver against the cluster solver (meshes of one CTA) and
 the streaming one (meshes beyond a cluster).  The streaming solver, which large and flat
 meshes still take, against the oracle, and its grid barrier's wait running out."""
+import time
+
 import numpy as np
 import pytest
 
@@ -101,3 +103,24 @@ def test_same_fp64_bits_from_every_solver_and_cut(monkeypatch, ncell, periodic, 
         out, it = on.smooth(phi[:nf])
         np.testing.assert_array_equal(out, want[:nf])
         np.testing.assert_array_equal(it, steps[:nf])
+
+
+def test_chip_is_cut_for_the_fields_asked_for():
+    """FP64 on 64 x 32 x 64: seven fields side by side take a seventh of the chip each, so one
+    field alone on such a seventh would take as long as seven, and eight twice as long.
+    Cut for its own number a call measured 0.23 and 1.23 times the time of seven."""
+    h = sedi.Sedi(dict(mesh((64, 32, 64), (1, 1, 0)), precision_form="fp64"))
+    x = torch.rand((8, h.C), dtype=torch.float64, device="cuda")
+    y = torch.empty_like(x)
+    it = np.zeros(8, np.int32)
+
+    def timed(nf):
+        t = []
+        for _ in range(6):
+            t0 = time.perf_counter()
+            h._check(sedi.lib().sedi_smooth(h.h, 0, nf, x.data_ptr(), y.data_ptr(), None, it.ctypes.data, 1))
+            t.append(time.perf_counter() - t0)
+        return float(np.median(t))
+
+    t1, t7, t8 = timed(1), timed(7), timed(8)
+    assert t1 <= 0.5 * t7 and t8 <= 1.6 * t7, (t1, t7, t8)
