@@ -2159,6 +2159,7 @@ struct RsPlan {
   int G = 0, px = 0, py = 0, pz = 0, groups = 0;
   int chunks = 0;             // of a thread
   size_t smem = 0, halo = 0;  // dynamic shared memory; halo words of a CTA and channel
+  double us = 0.0;            // predicted time of a step of all fields
 };
 
 // Bytes of a group's tagged words: the sums, and for each CTA two parities of the halo words
@@ -2216,6 +2217,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
       best.chunks = chunks;
       best.smem = smem;
       best.halo = halo;
+      best.us = cost;
     }
   };
   if (rs_one_cta(form, m)) {
@@ -2229,6 +2231,42 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
       for (int py = 1; py * pz <= gmax; ++py) consider(gmax / (py * pz), py, pz, g);
   }
   return best;
+}
+
+// Which FP64 meshes of a batch share a launch of the streaming solver (plan.G = 0) and which
+// have the chip to themselves one after the other.  In microseconds a step, fitted to
+// ensembles of equal beds, seven fields: the streaming solver takes 2 + 21 for every unit an SM has,
+// one at least; a mesh on chip what its plan says and 3 for each wave of its fields.  Small
+// meshes leave the chip to the latency of the exchange: 256 beds of 8^3 cells 178 ms on
+// chip, 10.4 streamed, 64 of 16^3 43.0 and 17.2, 8 of 19 x 15 x 31 6.4 and 5.4; 2 of those
+// 1.7 and 5.4, 4 of 48^3 17.4 and 28.7.  Small meshes are not planned where a bound of their time, their
+// cells over the whole chip and the latency, settles it.
+template <class Item>
+void fp64_batch_plans(std::vector<Item>& items, int nf, int nsm) {
+  auto stream_us = [&](int64_t units) { return 2.0 + 21.0 * std::max(1.0, (double)units / nsm); };
+  auto plan = [&](Item& it) {
+    it.pl = rs_plan(FORM_FP64, it.m, nf, nsm);
+    return it.pl.G ? it.pl.us + 3.0 * ((nf + it.pl.groups - 1) / it.pl.groups) : 1e300;
+  };
+  std::vector<Item*> rest;  // not worth the chip beside a streaming launch that is full
+  double sum = 0.0;
+  int64_t units = 0;
+  std::vector<Item*> open;  // of those, not planned yet
+  for (Item& it : items) {
+    const double share = 21.0 * (double)it.m.nu / nsm, bound = 4.5 + 0.006 * (double)it.m.C * nf / nsm;
+    const double t = bound < share ? plan(it) : bound;
+    if (bound >= share) open.push_back(&it);
+    if (t < share) continue;
+    rest.push_back(&it);
+    sum += t;
+    units += it.m.nu;
+  }
+  if (rest.empty()) return;
+  if (sum < stream_us(units)) {
+    for (Item* it : open) sum += plan(*it) - (4.5 + 0.006 * (double)it->m.C * nf / nsm);
+    if (sum < stream_us(units)) return;
+  }
+  for (Item* it : rest) it->pl = RsPlan{};
 }
 
 // The fields of one mesh over the groups of a cooperative launch (every CTA resident, one
@@ -2279,18 +2317,24 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
   // 440 us in a cluster solver's CTA, 250 here), larger meshes that fit a cluster's shared
   // memory the cluster solver (one launch for every mesh of a cluster size), still larger
   // ones the resident solver again where a cut of the whole chip fits, else the streaming grid
-  // solver.  In FP64 there is no cluster solver.  No bit of a result depends on the choice.
+  // solver.  In FP64 there is no cluster solver (several meshes: fp64_batch_plans).  No bit of a
+  // result depends on the choice.
   struct Item {
     SmoothMeshDev m;
     RsPlan pl;
   };
   std::vector<SmoothMeshDev> mg, mc;
   std::vector<Item> mr;
+  std::vector<Item> all(B);
   for (int b = 0; b < B; ++b) {
-    Item it;
+    Item& it = all[b];
     smooth_mesh_layout(form, scheme, meshes[b], &it.m);
     cluster_plan(form, it.m, &it.m.cl_size, &it.m.cl_planes);
-    if (resident && (it.m.cl_size == 0 || rs_one_cta(form, it.m))) it.pl = rs_plan(form, it.m, nf, nsm);
+    if (resident && (it.m.cl_size == 0 ? form != FORM_FP64 || B == 1 : rs_one_cta(form, it.m)))
+      it.pl = rs_plan(form, it.m, nf, nsm);
+  }
+  if (resident && form == FORM_FP64 && B > 1) fp64_batch_plans(all, nf, nsm);
+  for (Item& it : all) {
     if (it.m.cl_size > 0 && it.pl.G != 1) {
       mc.push_back(it.m);
     } else if (it.pl.G > 0) {
