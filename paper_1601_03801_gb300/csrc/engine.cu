@@ -51,6 +51,8 @@ struct sedi_handle {
   Block part_block;                // per-particle buffers
   Block bin_block;                 // link-cell bins (resized when the bin size changes)
   std::vector<void*> mesh_allocs;
+  Block tag_block;                 // the smoother's tagged words (see smooth_tags)
+  Block* tags = &tag_block;        // a bed: its ensemble's
   double rc_max = 0.0;             // largest list cutoff 2 r_max (1 + f) + skin
   int64_t since_set = 0;               // substeps since the particles were set
   bool is_bed = false;                 // a bed of an ensemble (stepped by the ensemble)
@@ -1102,9 +1104,21 @@ void sedi_default_params(sedi_params* p) {
   p->cnn_scale[0] = p->cnn_scale[1] = p->cnn_scale[2] = p->cnn_scale[3] = 1.0;
 }
 
+static int create_handle(const sedi_params* p, sedi_handle* of, sedi_handle** out, int bed = 0);
+
+static bool tags_in_work(const sedi_handle* h) {
+  return h->tags == &h->tag_block && smooth_beyond_cluster(h->P.C);
+}
+
 int sedi_create(const sedi_params* p, sedi_handle** out) {
   if (!p || !out) return SEDI_EINVAL;
   *out = nullptr;
+  return create_handle(p, nullptr, out);
+}
+
+// A handle, or a bed of the ensemble `of`: on its stream, with its status slot `bed` and
+// its room for tagged words.
+static int create_handle(const sedi_params* p, sedi_handle* of, sedi_handle** out, int bed) {
   sedi_handle* h = new sedi_handle();
   h->prm = *p;
   int rc = check_params(h, *p);
@@ -1157,7 +1171,8 @@ int sedi_create(const sedi_params* p, sedi_handle** out) {
     sedi_destroy(h);
     return rc;
   }
-  h->work_bytes = smooth_work_bytes(h->form, C, 8, h->prm.tau_scheme);
+  if (of) h->tags = &of->tag_block;
+  h->work_bytes = smooth_work_bytes(h->form, C, 8, h->prm.tau_scheme, tags_in_work(h));
   if ((rc = dmalloc(h, h->mesh_allocs, &h->work, h->work_bytes))) {
     sedi_destroy(h);
     return rc;
@@ -1176,15 +1191,16 @@ int sedi_create(const sedi_params* p, sedi_handle** out) {
       sedi_destroy(h);
       return SEDI_ENOMEM;
     }
-    for (int b = 0; b < p->n_beds; ++b) {
-      if ((rc = sedi_create(&q, &h->beds[b]))) {
+    for (int b = 0; b < p->n_beds; ++b)
+      if ((rc = create_handle(&q, h, &h->beds[b], b))) {
         sedi_destroy(h);
         return rc;
       }
-      h->beds[b]->stream = h->stream;
-      h->beds[b]->is_bed = true;
-      h->beds[b]->ctl_host = h->ctl_pin + b;
-    }
+  }
+  if (of) {
+    h->stream = of->stream;
+    h->is_bed = true;
+    h->ctl_host = of->ctl_pin + bed;
   }
   *out = h;
   return 0;
@@ -1205,6 +1221,7 @@ void sedi_destroy(sedi_handle* h) {
     if (p) cudaFree(p);
   for (cudaEvent_t e : h->avg_ev) cudaEventDestroy(e);
   if (h->part_block.p) cudaFree(h->part_block.p);
+  if (h->tag_block.p) cudaFree(h->tag_block.p);
   if (h->ctl_pin) cudaFreeHost(h->ctl_pin);
   if (h->bin_block.p) cudaFree(h->bin_block.p);
   if (h->ens_side.fork) cudaEventDestroy(h->ens_side.fork);
@@ -1248,11 +1265,8 @@ int sedi_set_bed(sedi_handle* h, int32_t bed, const double lo[3], const double h
     q.ncell[a] = ncell[a];
   }
   sedi_handle* nb = nullptr;
-  const int rc = sedi_create(&q, &nb);
+  const int rc = create_handle(&q, h, &nb, bed);
   if (rc) return fail(h, rc, "bed %d: invalid box or mesh", bed);
-  nb->stream = h->stream;
-  nb->is_bed = true;
-  nb->ctl_host = h->ctl_pin + bed;
   sedi_handle* old = h->beds[bed];
   old->stream = old->own;
   cudaStreamSynchronize(h->stream);
@@ -1454,6 +1468,23 @@ static int deposit_dev(sedi_handle* h) {
   return 0;
 }
 
+// The smoother's room for tagged words: behind the direction arrays for the mesh of a handle
+// beyond a cluster; shared by the beds of an ensemble (256 FP64 beds with 4 MB each held
+// 1 GB), and allocated by the first smoothing for FP64 meshes, since a small handle is created
+// in 0.3 ms without it and 0.4 with.  Without the room a mesh is streamed, to the same bits.
+static SmoothTags smooth_tags(sedi_handle* h) {
+  if (tags_in_work(h)) return {};
+  Block& b = *h->tags;
+  const size_t n = smooth_tag_room(h->form, h->P.C);
+  if (b.n < n) {
+    if (b.p) cudaFree(b.p);  // waits for the launches that use it
+    b = Block{};
+    if (cudaMalloc((void**)&b.p, n) == cudaSuccess) b.n = n;
+    else b.p = nullptr, cudaGetLastError();
+  }
+  return {false, b.p, (int64_t)b.n};
+}
+
 static int smooth_dev(sedi_handle* h, int nf, const void* guess, int n_tau = -1, bool zero_iters = true) {
   if (zero_iters) CK(cudaMemsetAsync(h->iters_dev, 0, 4 * 8, h->stream));
   // FP32 words cannot reach a relative residual much below 1e-6
@@ -1461,7 +1492,7 @@ static int smooth_dev(sedi_handle* h, int nf, const void* guess, int n_tau = -1,
   int rc = launch_smooth(h->form, h->P, h->phi, guess, nf, h->work, h->st, h->iters_dev,
                          rtol, h->prm.cg_max_iter, n_tau > 0 ? n_tau : h->prm.n_tau,
                          h->prm.tau_scheme, h->coef, h->P.graded ? &h->zs : nullptr,
-                         h->stream, h->barrier_spins, h->smooth_resident);
+                         h->stream, h->barrier_spins, h->smooth_resident, smooth_tags(h));
   if (rc) return fail(h, SEDI_ECUDA, "cooperative launch of the smoother failed: %s", cudaGetErrorString(cudaGetLastError()));
   return 0;
 }
@@ -1913,8 +1944,6 @@ static int ens_step(sedi_handle* h, int n) {
   return 0;
 }
 
-// Deposition and smoothing of every bed in batched launches; the smoothed eps
-// feeds each bed's drag.  Outputs stay on the device.
 static int ens_streams(sedi_handle* h) {
   if (h->ens_side_set) return 0;
   SmoothSide& e = h->ens_side;
@@ -1927,6 +1956,8 @@ static int ens_streams(sedi_handle* h) {
   return 0;
 }
 
+// Deposition and smoothing of every bed in batched launches; the smoothed eps
+// feeds each bed's drag.  Outputs stay on the device.
 static int ens_average(sedi_handle* h) {
   int rc = ens_finalize(h);
   if (rc) return rc;
@@ -1941,12 +1972,14 @@ static int ens_average(sedi_handle* h) {
   launch_deposit_ens(h->form, h->ens, h->stream);
   if (h->prm.profile) CK(cudaEventRecord(h->avg_ev[1], h->stream));
   std::vector<SmoothMesh> m(B);
+  for (sedi_handle* sb : h->beds) smooth_tags(sb);  // the room for the largest need
   for (int b = 0; b < B; ++b) {
     sedi_handle* sb = h->beds[b];
     SmoothMesh& x = m[b];
     x.phi = sb->phi;
     x.guess = nullptr;
     x.work = sb->work;
+    x.tags = smooth_tags(sb);
     x.iters = h->ens_iters + 8 * b;
     x.C = sb->P.C;
     x.nf = 7;

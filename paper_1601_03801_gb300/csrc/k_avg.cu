@@ -528,7 +528,7 @@ constexpr int64_t kStaticWords = SEDI_STATIC_MAX_WORDS;
 // 8 * cells <= kStaticWords (n_fields <= 8).  Upper bound of the solver scratch then
 // (FP64 form with BDF2, the largest case): the wide right-hand side and the BDF2
 // previous step (n_fields * cells <= kStaticWords words of 8 bytes each), three
-// narrow [cells][8] arrays (8-byte words) and the FP64 form's tagged words, kSmoothSums per-unit sums of every field
+// narrow [cells][8] arrays (8-byte words) and room for tagged words, kSmoothSums per-unit sums of every field
 // for up to kStaticWords / (8 * 256) + 1 units of 256 cells, the unit table (4 bytes a
 // unit), and 64 KB for the batch tables of one mesh and the 256-byte alignment of
 // each part.

@@ -1586,8 +1586,8 @@ __global__ void __launch_bounds__(kRsThreads, 1) k_smooth_rs(SmoothBatchDev a) {
       s_g.xp = md.xp ? (T*)md.xp + f * C : nullptr;
       s_g.guess = md.guess ? (const T*)md.guess + f * C : nullptr;
       s_g.r = G == 1 ? (N*)(s_pull + nu_max) : (N*)md.q + f * C;
-      s_g.sums = (unsigned long long*)md.d[0] + (size_t)grp * rs_sum_words(G);
-      s_g.halo = (unsigned long long*)md.d[0] + (size_t)ngrp * rs_sum_words(G) + (size_t)grp * G * 2 * P::n * hw * NW;
+      s_g.sums = (unsigned long long*)md.tags + (size_t)grp * rs_sum_words(G);
+      s_g.halo = (unsigned long long*)md.tags + (size_t)ngrp * rs_sum_words(G) + (size_t)grp * G * 2 * P::n * hw * NW;
     }
     __syncthreads();
 #pragma unroll 1
@@ -1985,35 +1985,46 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 int64_t smooth_units(int64_t C) { return (C + kThreads - 1) / kThreads; }
 
-// Room for the resident solver's tagged words behind the direction arrays: what these lack
-// of 24 MB for meshes beyond a cluster (150 CTAs of 160 KB), 4 MB for the small meshes of
-// the FP64 form.
-static size_t rs_extra(int form, int64_t C) {
+bool smooth_beyond_cluster(int64_t C) { return C > (int64_t)kClMaxCta * kClCells; }
+
+// What the direction arrays lack of 24 MB for meshes beyond a cluster (150 CTAs of 160 KB).  The
+// small meshes of the FP64 form: seven groups of 21 CTAs use 0.35 MB and 30 to 60 KB for each
+// cell of a brick's face, up to 4 MB more than their arrays hold; flat ones more, and take
+// another cut.
+size_t smooth_tag_bytes(int form, int64_t C) {
   const size_t have = 2 * align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4)), want = 24 << 20;
-  if (C > (int64_t)kClMaxCta * kClCells) return have < want ? want - have : 0;
-  return form == FORM_FP64 ? (size_t)kSmoothTagBytes : 0;
+  if (smooth_beyond_cluster(C)) return have < want ? want - have : 0;
+  if (form != FORM_FP64) return 0;
+  const double face = std::cbrt((double)C / 21 * (double)C / 21);
+  return align256((size_t)std::min(0.4e6 + 60e3 * face, (double)kSmoothTagBytes - 256));
 }
 
-size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme) {
+size_t smooth_tag_room(int form, int64_t C) {
+  const size_t lack = smooth_tag_bytes(form, C);
+  return lack ? lack + 2 * align256((size_t)kMaxF * C * (form == FORM_FP64 ? 8 : 4)) : 0;
+}
+
+size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme, bool own_tags) {
   const size_t w = form == FORM_PLAIN ? 4 : 8;             // wide word
   const size_t n = form == FORM_FP64 ? 8 : 4;              // narrow word
   const size_t wide = align256((size_t)nf * C * w);        // b, and x^{m-1} for BDF2
-  return (scheme == TAU_BDF2 ? 2 : 1) * wide + 3 * align256((size_t)kMaxF * C * n) + rs_extra(form, C) +
-         align256((size_t)smooth_units(C) * kMaxF * kQ * 8) + 256;
+  return (scheme == TAU_BDF2 ? 2 : 1) * wide + 3 * align256((size_t)kMaxF * C * n) +
+         (own_tags ? smooth_tag_bytes(form, C) : 0) + align256((size_t)smooth_units(C) * kMaxF * kQ * 8) + 256;
 }
 
-size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme) {
-  return align256(smooth_mesh_bytes(form, C, nf, scheme)) + smooth_batch_bytes(1, smooth_units(C));
+size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme, bool own_tags) {
+  return align256(smooth_mesh_bytes(form, C, nf, scheme, own_tags)) + smooth_batch_bytes(1, smooth_units(C));
 }
 
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf, void* work,
                   const DevState& st, int* iters_dev, double rtol, int max_iter, int n_tau,
                   int scheme, const double coef[3], const SmoothZ* z, cudaStream_t s,
-                  long long spin_limit, bool resident) {
+                  long long spin_limit, bool resident, const SmoothTags& tags) {
   SmoothMesh m{};
   m.phi = phi;
   m.guess = guess;
   m.work = work;
+  m.tags = tags;
   m.iters = iters_dev;
   m.C = P.C;
   m.nf = nf;
@@ -2023,7 +2034,7 @@ int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, in
     m.coef[k] = coef[k];
   }
   if (z) m.z = *z;
-  void* batch = (char*)work + align256(smooth_mesh_bytes(form, P.C, nf, scheme));
+  void* batch = (char*)work + align256(smooth_mesh_bytes(form, P.C, nf, scheme, tags.own));
   return launch_smooth_batch(form, &m, 1, nf, batch, rtol, max_iter, n_tau, scheme, st.ctl,
                              1 << 30, s, spin_limit, nullptr, resident);
 }
@@ -2081,8 +2092,15 @@ static void smooth_mesh_layout(int form, int scheme, const SmoothMesh& in, Smoot
   m.q = p;
   m.d[0] = p + nar;
   m.d[1] = p + 2 * nar;
-  m.halo_bytes = (int64_t)(2 * nar + rs_extra(form, in.C));
-  p += 3 * nar + rs_extra(form, in.C);
+  // tagged words from d[0] on: a resident launch has no other use for the direction arrays
+  const size_t extra = in.tags.own ? smooth_tag_bytes(form, in.C) : 0;
+  m.tags = m.d[0];
+  m.tag_bytes = (int64_t)(2 * nar + extra);
+  if (!in.tags.own && in.tags.n > m.tag_bytes) {
+    m.tags = in.tags.p;
+    m.tag_bytes = in.tags.n;
+  }
+  p += 3 * nar + extra;
   m.part = (double*)p;
   m.iters = in.iters;
   m.C = in.C;
@@ -2201,9 +2219,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
     const double units = 2.0 * (double)(nzc * (bx + by)), planes = zcut ? 2.0 * (double)(bx * by) : 0.0;
     double t = word == 8 ? 0.006 * (double)(nch * kRsZ) : 0.45 * chunks;
     if (G > 1) {
-      // every group's tagged sums and halo words live in the direction arrays of the
-      // mesh's scratch
-      if ((int64_t)rs_tag_bytes(G, halo) * groups > m.halo_bytes) return;
+      if ((int64_t)rs_tag_bytes(G, halo) * groups > m.tag_bytes) return;
       t += 1.5 + 0.0018 * units + 0.00015 * planes;
     }
     const double cost = t * ((nf + groups - 1) / groups);  // waves of the fields
@@ -2288,7 +2304,7 @@ int launch_rs(const SmoothBatchDev& a, const RsPlan& pl, const SmoothMeshDev& m,
   if ((int64_t)per_sm * nsm < (int64_t)pl.groups * pl.G) return -3;
   // no tagged word of an earlier launch may pass for this one's: exchanges count from 1
   const size_t bytes = rs_tag_bytes(pl.G, pl.halo) * pl.groups;
-  if (cudaMemsetAsync(m.d[0], 0, bytes, s) != cudaSuccess) return -3;
+  if (cudaMemsetAsync(m.tags, 0, bytes, s) != cudaSuccess) return -3;
   SmoothBatchDev args = a;
   void* p[] = {&args};
   return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)(pl.groups * pl.G)), dim3(kRsThreads), p, pl.smem, s) ==

@@ -154,11 +154,20 @@ struct SmoothZ {
   double zmax[2];
 };
 
+// Room for the resident solver's tagged words: a part of a mesh's own scratch, or memory that
+// the meshes of one stream share (their launches follow each other).
+struct SmoothTags {
+  bool own = true;
+  void* p = nullptr;
+  int64_t n = 0;
+};
+
 // One mesh of a smoothing batch, as the caller describes it.
 struct SmoothMesh {
   void* phi;          // [nf][C] fields in the smoothing word of the form, in place
   const void* guess;  // [nf][C] initial guess of the first pseudo-step, or null
-  void* work;         // smooth_mesh_bytes(form, C, nf, scheme) bytes of device scratch
+  void* work;         // smooth_mesh_bytes(form, C, nf, scheme, tags.own) bytes of device scratch
+  SmoothTags tags;
   int* iters;         // [nf] device counters, incremented by the steps taken (or null)
   int64_t C;
   int32_t nc[3], per[3];
@@ -193,7 +202,8 @@ struct alignas(16) SmoothMeshDev {
   int32_t nc[3], per[3];
   uint64_t div_x, div_xy;            // ceil(2^64 / nx), ceil(2^64 / (nx ny)) (0: divisor 1)
   int32_t cl_size, cl_planes;        // cluster solver's CTAs, z-planes per CTA (0: does not fit)
-  int64_t halo_bytes;                // resident solver: room for halo words from d[0] on
+  void* tags;                        // resident solver: tagged words, and the room for them
+  int64_t tag_bytes;
   int32_t rs_G, rs_px, rs_py, rs_pz;  // resident solver: CTAs, cuts per axis (0: streaming solver)
   SmoothSpec sp[2];  // [0]: backward-Euler steps (coef); [1]: BDF2 steps (2/3 coef)
   SmoothZ z;         // graded z mesh (null: uniform)
@@ -225,7 +235,7 @@ constexpr long long kBarrierSpins = 1ll << 22;
 constexpr int kSmoothUnitCells = 256;
 constexpr int kSmoothMaxFields = 8;
 constexpr int kSmoothSums = 4;
-// the resident solver's tagged words of a small FP64 mesh (see smooth_mesh_bytes)
+// smooth_tag_bytes of a mesh that fits a cluster at most
 constexpr int kSmoothTagBytes = 4 << 20;
 
 // Streams beside the caller's for the launches of a batch, and their events.
@@ -236,8 +246,13 @@ struct SmoothSide {
 };
 
 int64_t smooth_units(int64_t C);
-// scratch of one mesh, and of the batch tables
-size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme);
+// scratch of one mesh (without own_tags: smooth_tag_bytes less), and of the batch tables
+size_t smooth_mesh_bytes(int form, int64_t C, int nf, int scheme, bool own_tags = true);
+// what a mesh's direction arrays lack of the room that the resident solver's tagged words use
+size_t smooth_tag_bytes(int form, int64_t C);
+// that room as a whole, for meshes that share it (0: the direction arrays will do)
+size_t smooth_tag_room(int form, int64_t C);
+bool smooth_beyond_cluster(int64_t C);
 size_t smooth_batch_bytes(int64_t B, int64_t U);
 // Smooth every mesh's nf fields in place by n_tau pseudo-steps of the scheme;
 // batch_work: smooth_batch_bytes(B, sum of units) bytes.  resident = false keeps every mesh off
@@ -247,12 +262,13 @@ int launch_smooth_batch(int form, const SmoothMesh* meshes, int B, int nf, void*
                         double rtol, int max_iter, int n_tau, int scheme, Ctl* ctl,
                         int max_blocks, cudaStream_t s, long long spin_limit = kBarrierSpins,
                         const SmoothSide* side = nullptr, bool resident = true);
-// Single mesh: work holds smooth_work_bytes(form, C, nf, scheme) = mesh + batch scratch.
-size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme);
+// Single mesh: work holds smooth_work_bytes(form, C, nf, scheme, tags.own) = mesh + batch scratch.
+size_t smooth_work_bytes(int form, int64_t C, int nf, int scheme, bool own_tags = true);
 int launch_smooth(int form, const DevParams& P, void* phi, const void* guess, int nf,
                   void* work, const DevState& st, int* iters_dev, double rtol, int max_iter,
                   int n_tau, int scheme, const double coef[3], const SmoothZ* z,
-                  cudaStream_t s, long long spin_limit = kBarrierSpins, bool resident = true);
+                  cudaStream_t s, long long spin_limit = kBarrierSpins, bool resident = true,
+                  const SmoothTags& tags = {});
 void launch_average_out(int form, const void* phi, const DevParams& P, void* ufe, double* eps,
                         double* Us, double* F, cudaStream_t s);
 void launch_phi_convert(int form, const void* phi, double* out, int64_t n, int to_double,

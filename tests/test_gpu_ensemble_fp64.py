@@ -72,3 +72,34 @@ def test_many_small_beds_share_the_chip():
 
     t2, t64 = timed(2), timed(64)
     assert t64 <= 10.0 * t2, (t2, t64)
+
+
+def test_beds_share_the_room_for_tagged_words():
+    """64 beds of 8^3 cells hold about 0.5 MB each; room of its own made it 4.5 MB a bed."""
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    e = ensemble(beds([(8, 8, 8)] * 64))
+    e.average_inplace()
+    used = free - torch.cuda.mem_get_info()[0]
+    e.close()
+    assert used <= 64 * 2e6, used
+
+
+@pytest.mark.parametrize("form", ["fp64", "split", "plain"])
+def test_a_bed_smooths_as_a_handle_does(form):
+    """Fields of a caller through a bed, whose room for tagged words is the ensemble's and grows
+    with later beds, and through a handle."""
+    prm = dict(default_params(), precision_form=form)
+    e = sedi.Sedi(dict(prm, n_beds=3))
+    meshes = [(8, 9, 7), (19, 15, 31), (53, 51, 49)]
+    for b, nc in enumerate(meshes):
+        hi = tuple(1e-3 * n for n in nc)
+        e.set_bed(b, (0.0, 0.0, 0.0), hi, nc)
+        for k in range(b + 1):
+            phi = np.random.default_rng(k).random((3, int(np.prod(meshes[k]))))
+            g = sedi.Sedi(dict(prm, hi=tuple(1e-3 * n for n in meshes[k]), ncell=meshes[k]))
+            out, it = e.smooth(phi, bed=k)
+            ref, ir = g.smooth(phi)
+            np.testing.assert_array_equal(out, ref)
+            np.testing.assert_array_equal(it, ir)
+            g.close()
