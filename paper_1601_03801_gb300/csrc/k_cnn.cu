@@ -47,8 +47,8 @@ __device__ __forceinline__ int64_t nb_of(const Grid3& g, int x, int y, int z) {
 // voxels that are staged with a halo of one voxel in shared memory: a tap is an offset
 // of the staged row, and every fragment is one ldmatrix of rows of 8 voxels along x.
 // FP32 gradients take part as three bf16 planes, the top, middle and low 8 bits of the
-// significand: their sum is the FP32 word, exactly, and so is each product with a bf16
-// weight or activation, so the operands are the FP32 ones.  The tensor cores' accumulation
+// significand: their sum is the FP32 word (see split3), and each product with a bf16
+// weight or activation is exact, so the operands are the FP32 ones.  The tensor cores' accumulation
 // does not round to nearest, so the top planes' products are summed in chains of two
 // instructions that are then added in FP32, and the lower planes' (2^-8 of them) apart.
 // The two layers whose outputs are rounded to bf16 keep one order of summation, tap after
@@ -108,7 +108,8 @@ __device__ __forceinline__ void mma_bf16_16816(float* c, const uint32_t* a, cons
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// g = p[0] + p[1] + p[2], exactly (infinities and NaN stay in p[0])
+// g = p[0] + p[1] + p[2], exactly from 2^-110 up (below, the low plane can lie under bf16's least
+// word, 2^-133); infinities and NaN stay in p[0]
 __device__ __forceinline__ void split3(float g, __nv_bfloat16* p) {
   const uint32_t u = __float_as_uint(g);
   if ((u & 0x7f800000u) == 0x7f800000u) {

@@ -742,6 +742,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
   const int64_t ncl = gridDim.x / csize, cid = blockIdx.x / csize;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t items = (int64_t)a.B * a.nf;
+  // one item a cluster as launched; the loop stays because the kernel without it is slower
+  // (four fields of 37 x 41 x 45 668 -> 680 us)
   for (int64_t w = cid; w < items; w += ncl) {
     const int bi = (int)(w / a.nf), f = (int)(w % a.nf);
     const SmoothMeshDev& md = a.mesh[bi];
