@@ -67,12 +67,13 @@ struct sedi_handle {
   int* iters_dev = nullptr;
   double* dstage = nullptr;  // [max(7C, 4*3N)] doubles
   size_t dstage_n = 0;
-  // copy of the control block: pinned memory (ctl_pin) in a handle that steps, and for all
-  // the beds of an ensemble at once, since that allocation costs 0.15 ms, a fifth of what a
-  // small handle takes to be created, loaded and released
+  // copy of the control block: pinned memory (ctl_pin, 3 us less a read) from the handle's
+  // eighth read on, and for all the beds of an ensemble at once, since that allocation costs
+  // 0.15 ms, a fifth of what a small handle takes to be created, loaded and released
   Ctl ctl_own{};
   Ctl* ctl_host = &ctl_own;
   Ctl* ctl_pin = nullptr;
+  int status_reads = 0;
   double coef[3] = {0, 0, 0};
   std::map<int, cudaGraphExec_t> graphs;
   sedi_stats stats{};
@@ -420,6 +421,10 @@ int ensure_stage(sedi_handle* h, size_t n) {
 // Read the device control block; map device-side errors to status codes.
 int sync_status(sedi_handle* h) {
   if (h->st.ctl) {
+    if (h->ctl_host == &h->ctl_own && ++h->status_reads == 8) {
+      if (cudaMallocHost((void**)&h->ctl_pin, sizeof(Ctl)) == cudaSuccess) h->ctl_host = h->ctl_pin;
+      else h->ctl_pin = nullptr, cudaGetLastError();
+    }
     CK(cudaMemcpyAsync(h->ctl_host, h->st.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream));
   }
   CK(cudaStreamSynchronize(h->stream));
@@ -647,10 +652,6 @@ int alloc_particles(sedi_handle* h, int64_t N, double rmax) {
 
 int build_graph(sedi_handle* h, int n, cudaGraphExec_t* out) {
   cudaGraph_t graph = nullptr;
-  if (!h->ctl_pin) {
-    CK(cudaMallocHost((void**)&h->ctl_pin, sizeof(Ctl)));
-    h->ctl_host = h->ctl_pin;
-  }
   sedi_handle::GraphEv ev;
   if (h->prm.profile)
     for (int s = 0; s < n; ++s) {
