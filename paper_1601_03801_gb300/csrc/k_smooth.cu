@@ -2202,6 +2202,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
   auto consider = [&](int px, int py, int pz, int groups) {
     if (px < 1 || px > nx || py > ny || pz > nz) return;
     const int G = px * py * pz;
+    if (G == 1 && !rs_one_cta(form, m)) return;  // a group (rs_sums); on a device of few SMs
     const int64_t bx = (nx + px - 1) / px, by = (ny + py - 1) / py, bz = (nz + pz - 1) / pz;
     const int64_t nzc = (bz + kRsZ - 1) / kRsZ, nch = bx * by * nzc;
     if (nch > top) return;
@@ -2209,7 +2210,7 @@ RsPlan rs_plan(int form, const SmoothMeshDev& m, int nf, int nsm) {
     const int64_t words = (nzc * (by + 2) * ((bx + 2) | 1) * kRsZ + (zcut ? 2 * bx * by : 0) + 3) / 4 * 4;
     const int64_t nu = 2 * nzc * (bx + by) + (zcut ? 2 * bx * by : 0);
     const size_t smem = (2 * (size_t)words + 2 * (size_t)nzc * kRsZ) * word + (size_t)nu * 12 +
-                        (G == 1 && word == 4 ? m.C * 4 : 0);
+                        (G == 1 ? m.C * 4 : 0);
     // a chunk's word holds 16 bits of index and 11 of its place along z
     if (smem > kRsSmem || words > 0xffff || nzc > 2000) return;
     const size_t halo = 2 * (size_t)(nzc * kRsZ * (bx + by) + (zcut ? bx * by : 0));
