@@ -1066,7 +1066,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_smooth_cl(SmoothBatchDev a) {
 // operation rate), one way between SMs through L2 for 0.8 us.
 // Seven fields of random values, microseconds a call, streaming grid solver -> here:
 // 128 x 64 x 128 9,760 -> 5,990, 256 x 128 x 64 10,190 -> 7,360, 96 x 96 x 24
-// 2,030 -> 1,140; 10 x 10 x 20 in one CTA 440 -> 250; FP64 19 x 15 x 31 4,390 -> 740 (the
+// 2,030 -> 1,140; 10 x 10 x 20 in one CTA 440 -> 250; FP64 19 x 15 x 31 4,390 -> 750 (the
 // streaming solver ran it on 35 blocks).
 constexpr int kRsZ = 4;              // cells of a chunk
 constexpr int kRsMaxGroup = 160;     // CTAs of a group at most
