@@ -634,8 +634,9 @@ def ensemble_leg(steps=3, warmup=2, settle=11):
             "speedup": round(ms_p / ms_b, 3),
             "launch_structure": "per fluid step: one CUDA graph of 20 substeps (a conditional "
                                 "batched rebuild node, then one batched substep launch over all "
-                                "beds, grid.y = bed), then one batched deposition and one "
-                                "persistent smoothing launch for all beds",
+                                "beds, grid.y = bed), then one batched deposition and the "
+                                "smoothing launches (one for each cluster size, one for all "
+                                "beds of one CTA)",
             "tuned": {"substep_variant": tuned["substep_variant"], "block": tuned["substep_block"],
                       "bins_per_cutoff": tuned["bins_per_cutoff"],
                       "bin_order": "xz"[tuned["bin_order"]] + " fastest", "settle_steps_untimed": settle},
