@@ -2,6 +2,7 @@
 // capture of the substep sequence (rebuild under a graph IF node decided on the
 // device), orchestration of the averaging, import/export in caller order and
 // checkpoints.  All arithmetic of the method runs in the kernels of k_*.cu.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <unistd.h>
 
@@ -391,9 +392,28 @@ int copy_out(sedi_handle* h, void* dst, const void* src, size_t bytes, int mem) 
   return 0;
 }
 
+// Whether `bytes` from `p` on lie in one allocation (false where that cannot be asked).
+bool in_allocation(const void* p, size_t bytes) {
+  using Get = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Get get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) ==
+                        cudaSuccess && r == cudaDriverEntryPointSuccess;
+    return ok ? (Get)f : nullptr;
+  }();
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[2] = {&start, &size};
+  if (!get || get(2, what, to, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+  return (CUdeviceptr)p >= start && (CUdeviceptr)p + bytes <= start + size;
+}
+
 // Where a kernel writes an output of the caller's: the output itself if it is memory of this
-// GPU, else the staging buffer, from which put_out copies it.
-double* out_at(double* out, double* stage, int mem) {
+// GPU, else the staging buffer, from which put_out copies it.  A buffer that is too small
+// goes to the copy, which refuses it; a kernel would write past its end.
+double* out_at(double* out, double* stage, size_t bytes, int mem) {
   if (!out || mem != SEDI_MEM_DEVICE || ((uintptr_t)out & 7)) return stage;
   int dev = 0;
   cudaPointerAttributes at{};
@@ -401,7 +421,7 @@ double* out_at(double* out, double* stage, int mem) {
     cudaGetLastError();
     return stage;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == dev ? out : stage;
+  return at.type == cudaMemoryTypeDevice && at.device == dev && in_allocation(out, bytes) ? out : stage;
 }
 
 int put_out(sedi_handle* h, double* out, const double* at, size_t bytes, int mem) {
@@ -2041,9 +2061,9 @@ static int ens_average(sedi_handle* h) {
 // Outputs of the last averaging of a single-bed handle (smoothing word -> FP64).
 static int average_outputs_dev(sedi_handle* h, double* eps, double* Us, double* F, int32_t mem) {
   const int64_t C = h->P.C;
-  double* const de = out_at(eps, h->dstage, mem);
-  double* const du = out_at(Us, h->dstage + C, mem);
-  double* const dF = out_at(F, h->dstage + 4 * C, mem);
+  double* const de = out_at(eps, h->dstage, 8 * C, mem);
+  double* const du = out_at(Us, h->dstage + C, 24 * C, mem);
+  double* const dF = out_at(F, h->dstage + 4 * C, 24 * C, mem);
   launch_average_out(h->form, h->phi, h->P, h->mesh.ufe, de, du, dF, h->stream);
   int rc;
   if ((rc = put_out(h, eps, de, 8 * C, mem)) || (rc = put_out(h, Us, du, 24 * C, mem)) ||
@@ -2309,7 +2329,7 @@ int sedi_get_particles(sedi_handle* h, int32_t bed, double* x, double* v, double
   double* outs[4] = {x, v, w, a};
   for (int k = 0; k < 4; ++k) {
     if (!outs[k]) continue;
-    double* const at = out_at(outs[k], h->dstage + 3 * N * k, mem);
+    double* const at = out_at(outs[k], h->dstage + 3 * N * k, 24 * N, mem);
     launch_export(h->form, h->st, k, at, h->stream);
     if ((rc = put_out(h, outs[k], at, 24 * N, mem))) return rc;
   }

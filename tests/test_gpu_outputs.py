@@ -1,5 +1,6 @@
 """Outputs into host arrays: the forces of few particles (one copy for the four arrays) and of
 more against device outputs, and large arrays whose pages the process has not touched."""
+import ctypes
 import time
 
 import numpy as np
@@ -63,3 +64,37 @@ def test_large_outputs_into_untouched_pages():
     f = h.compute_forces()
     for k, a in zip(("contact", "lub", "fluid", "torque"), out):
         np.testing.assert_array_equal(f[k], a)
+
+
+def test_device_output_that_is_too_small_is_refused():
+    """A device buffer smaller than the output is refused by the copy to it, as a host check: no
+    kernel writes past its end.  The bytes behind it, in the same 2 MB page, stay."""
+    cudart = ctypes.CDLL(next(line.split()[-1] for line in open("/proc/self/maps") if "libcudart.so" in line))
+
+    def malloc(size):
+        p = ctypes.c_void_p()
+        assert cudart.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0
+        return p.value
+
+    n = 1000
+    h = handle(n)
+    C = h.C
+    short = 24 * n - 8192
+    page = 2 << 20
+    p = malloc(short)
+    if p % page + 24 * n + 24 * C > page:
+        pytest.skip("the buffer ends its page")
+    for call in (lambda: sedi.lib().sedi_get_particles(h.h, 0, p, None, None, None, 1),
+                 lambda: sedi.lib().sedi_average(h.h, 0, None, p - p % 8 + short // 8 * 8 - 8, None, 1)):
+        with pytest.raises(sedi.SediError) as e:
+            h._check(call())
+        assert e.value.code == -3
+    h.step(2)  # the handle and the context are in order
+    want = h.get_particles()[0]
+    q = malloc(24 * n)
+    h._check(sedi.lib().sedi_get_particles(h.h, 0, q, None, None, None, 1))
+    got = np.zeros((n, 3))
+    assert cudart.cudaMemcpy(ctypes.c_void_p(got.ctypes.data), ctypes.c_void_p(q), ctypes.c_size_t(24 * n), 2) == 0
+    np.testing.assert_array_equal(got, want)
+    for r in (p, q):
+        cudart.cudaFree(ctypes.c_void_p(r))
